@@ -204,6 +204,8 @@ vktError launch_separable(const Job& job, const float* gx, const float* gy, cons
 vktError tensor_available(const vktStructuredVolume_impl* dst, const vktStructuredVolume_impl* src,
                           const vktFilter_impl* f);
 vktError launch_tensor(const Job& job, const float* w, int k, const Ctx& ctx);
+// Whether one tensor-core launch can take n volumes of the job's dims spaced vs voxels apart.
+bool tensor_batchable(const Job& job, int32_t n, int64_t vs);
 
 // Whether a separable filter into an integer destination needs compensated accumulation.
 bool separable_needs_comp(const vktStructuredVolume_impl* dst, const vktStructuredVolume_impl* src,

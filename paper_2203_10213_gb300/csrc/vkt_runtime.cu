@@ -875,8 +875,8 @@ static vktError apply_filter(vktStructuredVolume dst, vktStructuredVolume src, v
 
 // A batch of n triples that share one dense (or direct-forced) filter, with equal dims,
 // formats and value ranges: the direct path takes one launch over all n volumes when
-// sources and destinations are evenly spaced (else one launch per volume), the tensor path
-// one launch per volume; no graph is built, so a filter whose weights change from call to
+// sources and destinations are evenly spaced (else one launch per volume), and so does the
+// tensor path where one tensor map can describe the sources; no graph is built, so a filter whose weights change from call to
 // call (a training step) costs no recapture.  Sets *handled when the batch qualifies (and
 // returns the launches' error); otherwise the caller builds its general batch.
 }  // extern "C"
@@ -900,6 +900,12 @@ vktError vkt::apply_filter_multi(int32_t n, vktStructuredVolume* dst, vktStructu
         if (f->separable) return VKT_NO_ERROR;   // the persistent separable batch
         path = (f->k >= 5 && tensor_available(dst[0], src[0], f) == VKT_NO_ERROR) ? VKT_PATH_TENSOR
                                                                                   : VKT_PATH_DIRECT;
+        // at k = 5 the direct launch, whose smaller tiles fill the GPU better, is the faster one
+        // for volumes of a power of two (8 x 128^3: direct 92 us, tensor 124; 2 x 64^3: 20 and
+        // 28) and near it otherwise (4 x 132x100x96: 60 and 51); at k = 7 the tensor launch is
+        // (8 x 128^3: 326 and 137 us)
+        int64_t s = 0;
+        if (f->k == 5 && evenly_spaced(n, src, &s) && evenly_spaced(n, dst, &s)) path = VKT_PATH_DIRECT;
     }
     if (path == VKT_PATH_SEPARABLE) return VKT_NO_ERROR;
     if (path == VKT_PATH_TENSOR) {
@@ -924,16 +930,15 @@ vktError vkt::apply_filter_multi(int32_t n, vktStructuredVolume* dst, vktStructu
     double wsum = 0.0;
     for (int i = 0; i < f->k * f->k * f->k; ++i) wsum += f->w[i];
     epilogue(dst[0], src[0], wsum, &job);
-    if (path == VKT_PATH_DIRECT) {
-        job.comp = direct_needs_comp(dst[0], src[0], f) ? 1 : 0;
-        if (even) {
-            job.src = src[0]->data;
-            job.dst = dst[0]->data;
-            job.nvol = n;
-            job.vs_src = ss;
-            job.vs_dst = sd;
-            return launch_direct(job, f->w, f->k, ctx);
-        }
+    if (path == VKT_PATH_DIRECT) job.comp = direct_needs_comp(dst[0], src[0], f) ? 1 : 0;
+    if (even && (path == VKT_PATH_DIRECT || tensor_batchable(job, n, ss))) {
+        job.src = src[0]->data;
+        job.dst = dst[0]->data;
+        job.nvol = n;
+        job.vs_src = ss;
+        job.vs_dst = sd;
+        return path == VKT_PATH_TENSOR ? launch_tensor(job, f->w, f->k, ctx)
+                                       : launch_direct(job, f->w, f->k, ctx);
     }
     for (int32_t i = 0; i < n && err == VKT_NO_ERROR; ++i) {
         job.src = src[i]->data;

@@ -15,6 +15,9 @@
 // the epilogue scales back and adds the k slot columns into k rotating register
 // accumulators, one of which completes per input plane (z-march).
 //
+// The items of a launch may span nvol volumes of equal dims (a training batch): one 128^3 volume
+// has too few of them to give every SM one, eight have.
+//
 // Warp roles (448 threads, one CTA per SM, persistent over (x, y, z-chunk) work items):
 //   warp 0       TMEM allocation; lane 0 issues TMA loads of f32 plane tiles
 //   warp 1       lane 0 issues the MMAs and commits
@@ -81,7 +84,8 @@ struct TcW {
 struct TcArgs {
     float* dst;
     int nx, ny, nz;
-    int items_x, items_y, items_z, nitems, zchunk;
+    int items_x, items_y, items_z, nitems, zchunk;   // items: x, then y, then z, then volume
+    int64_t vs_dst;      // voxels from one volume's destination to the next
     int wexp;            // weights are scaled by 2^wexp before splitting
     unsigned* status;
 };
@@ -270,7 +274,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             bool ok = true;
             for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
                 const int xi = item % p.items_x, yi = (item / p.items_x) % p.items_y;
-                const int zi = item / (p.items_x * p.items_y);
+                const int zv = item / (p.items_x * p.items_y);
+                const int vol = zv / p.items_z, zi = zv - vol * p.items_z;
                 const int x0 = xi * 8 * XT, y0 = yi * MROWS, zc0 = zi * p.zchunk;
                 const int zc1 = min(zc0 + p.zchunk, p.nz);
                 const int nplanes = zc1 - zc0 + 2 * R;
@@ -282,8 +287,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                         break;
                     }
                     mbar_arrive_expect_tx(&h.stage_full[s], C::STAGE_TX);
-                    tma_load_3d(smem + C::OFF_STAGE + s * C::STAGE_BYTES, &tmap, &h.stage_full[s],
-                                x0 - 4, y0 - R, clampi(zc0 - R + it, 0, p.nz - 1));
+                    tma_load_4d(smem + C::OFF_STAGE + s * C::STAGE_BYTES, &tmap, &h.stage_full[s],
+                                x0 - 4, y0 - R, clampi(zc0 - R + it, 0, p.nz - 1), vol);
                 }
             }
             // drain: every issued load completes its stage (bounded, no abort check)
@@ -320,7 +325,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             uint32_t g = 0;
             bool ok = true;
             for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
-                const int zi = item / (p.items_x * p.items_y);
+                const int zi = item / (p.items_x * p.items_y) % p.items_z;
                 const int zc0 = zi * p.zchunk, zc1 = min(zc0 + p.zchunk, p.nz);
                 const int nplanes = zc1 - zc0 + 2 * R;
                 for (int it = 0; it < nplanes; ++it, ++g) {
@@ -368,7 +373,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         uint32_t g = 0;
         for (int item = blockIdx.x; item < p.nitems; item += gridDim.x) {
             const int xi = item % p.items_x, yi = (item / p.items_x) % p.items_y;
-            const int zi = item / (p.items_x * p.items_y);
+            const int zi = item / (p.items_x * p.items_y) % p.items_z;
             const int x0 = xi * 8 * XT, y0 = yi * MROWS, zc0 = zi * p.zchunk;
             const int zc1 = min(zc0 + p.zchunk, p.nz);
             const int nplanes = zc1 - zc0 + 2 * R;
@@ -466,7 +471,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         bool ok = true;
         for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
             const int xi = item % p.items_x, yi = (item / p.items_x) % p.items_y;
-            const int zi = item / (p.items_x * p.items_y);
+            const int zv = item / (p.items_x * p.items_y);
+            const int vol = zv / p.items_z, zi = zv - vol * p.items_z;
+            float* const dst = p.dst + vol * p.vs_dst;
             const int x0 = xi * 8 * XT, y0 = yi * MROWS, zc0 = zi * p.zchunk;
             const int zc1 = min(zc0 + p.zchunk, p.nz);
             const int nplanes = zc1 - zc0 + 2 * R;
@@ -513,7 +520,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 const int sl0 = ((u - R) % K + K) % K;
                 if (it >= 2 * R && oy < p.ny && nvalid > 0) {
                     const int oz = zc0 + it - 2 * R;
-                    float* d = p.dst + (static_cast<int64_t>(oz) * p.ny + oy) * p.nx + ox;
+                    float* d = dst + (static_cast<int64_t>(oz) * p.ny + oy) * p.nx + ox;
                     if (nvalid >= 8 && ((reinterpret_cast<uintptr_t>(d) & 15) == 0)) {
                         reinterpret_cast<float4*>(d)[0] = make_float4(acc[sl0][0], acc[sl0][1], acc[sl0][2], acc[sl0][3]);
                         reinterpret_cast<float4*>(d)[1] = make_float4(acc[sl0][4], acc[sl0][5], acc[sl0][6], acc[sl0][7]);
@@ -573,16 +580,18 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     a.items_x = (job.nx + 8 * XT - 1) / (8 * XT);
     a.items_y = (job.ny + MROWS - 1) / MROWS;
+    const int nvol = std::max(job.nvol, 1);
     const long xy = static_cast<long>(a.items_x) * a.items_y;
-    // enough z chunks for ~6 items per SM, but chunks of at least 8 r planes
-    long chunks = std::max<long>(1, (6L * sms + xy - 1) / xy);
-    chunks = std::min<long>(chunks, std::max(1, job.nz / std::max(8, 8 * C::R)));
-    a.zchunk = static_cast<int>((job.nz + chunks - 1) / chunks);
+    // whole waves of one CTA per SM over all volumes' items, counting each chunk's halo planes
+    a.zchunk = zchunk_waves(xy * nvol, job.nz, sms, C::R);
     a.items_z = (job.nz + a.zchunk - 1) / a.zchunk;
-    a.nitems = static_cast<int>(xy * a.items_z);
+    if (xy * a.items_z > 0x7fffffff / nvol) return VKT_ERROR_UNSUPPORTED;
+    a.nitems = static_cast<int>(xy * a.items_z * nvol);
+    a.vs_dst = job.vs_dst;
 
     alignas(64) CUtensorMap map;
-    if (!encode_tensor_map_3d(&map, FMT_F32, job.src, job.nx, job.ny, job.nz, NCH * 8, C::ROWS, 1))
+    if (!encode_tensor_map(&map, FMT_F32, job.src, job.nx, job.ny, job.nz, nvol, job.vs_src, NCH * 8,
+                           C::ROWS, 1))
         return VKT_ERROR_UNSUPPORTED;
     cudaError_t e = cudaFuncSetAttribute(k_tc<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return from_cuda(e);
@@ -606,6 +615,13 @@ vktError tensor_available(const vktStructuredVolume_impl* dst, const vktStructur
     if (src->dims[0] % 4 != 0 || reinterpret_cast<uintptr_t>(src->data) % 16 != 0)
         return VKT_ERROR_UNSUPPORTED;   // rows must be describable by a TMA tensor map
     return VKT_NO_ERROR;
+}
+
+bool tensor_batchable(const Job& job, int32_t n, int64_t vs)
+{
+    // the tensor map's volume stride is a multiple of 16 bytes, and the items are counted in 31 bits
+    const int64_t items = static_cast<int64_t>((job.nx + 15) / 16) * ((job.ny + MROWS - 1) / MROWS) * job.nz;
+    return (vs * 4) % 16 == 0 && items <= 0x7fffffff / n;
 }
 
 vktError launch_tensor(const Job& job, const float* w, int k, const Ctx& ctx)
