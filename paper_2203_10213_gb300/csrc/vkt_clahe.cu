@@ -355,15 +355,11 @@ extern "C" vktError vktClahe3DSV(vktStructuredVolume dst, vktStructuredVolume sr
         limit = static_cast<int64_t>(std::floor(static_cast<double>(clipLimit) * static_cast<double>(n) / 256.0));
         limit = std::max<int64_t>(limit, 1);
     }
+    // one block of scratch: the histograms, then the mappings
     unsigned* hist = nullptr;
-    uint8_t* luts = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&hist), nbricks * 256 * sizeof(unsigned), ctx.stream);
-    if (e != cudaSuccess) return from_cuda(e);
-    e = cudaMallocAsync(reinterpret_cast<void**>(&luts), nbricks * 256, ctx.stream);
-    if (e != cudaSuccess) {
-        cudaFreeAsync(hist, ctx.stream);
-        return from_cuda(e);
-    }
+    err = scratch_alloc(reinterpret_cast<void**>(&hist), nbricks * 256 * (sizeof(unsigned) + 1), ctx);
+    if (err != VKT_NO_ERROR) return err;
+    uint8_t* luts = reinterpret_cast<uint8_t*>(hist + nbricks * 256);
     const uint8_t* s = static_cast<const uint8_t*>(src->data);
     // widest loads the rows allow (brick rows and volume rows multiples of the width, the
     // data 16-byte aligned)
@@ -393,14 +389,13 @@ extern "C" vktError vktClahe3DSV(vktStructuredVolume dst, vktStructuredVolume sr
         k_clahe_map<<<grid, NT, 0, ctx.stream>>>(s, g, luts, static_cast<uint8_t*>(dst->data));
     }
     count_launches(3);
-    e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
     if (ctx.debug & VKT_DEBUG_LOG)
         fprintf(stderr, "[vkt] clahe3d %dx%dx%d bricks %dx%dx%d (%dx%dx%d voxels) limit=%lld blend=%s\n",
                 g.nx, g.ny, g.nz, bricksX, bricksY, bricksZ, g.sx, g.sy, g.sz,
                 static_cast<long long>(limit), by_cells ? "cells" : "voxels");
     if (ctx.debug & VKT_DEBUG_LOG) fprintf(stderr, "[vkt] clahe3d histogram loads of %d bytes\n", vec);
     const cudaError_t e1 = cudaFreeAsync(hist, ctx.stream);
-    const cudaError_t e2 = cudaFreeAsync(luts, ctx.stream);
-    if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2;
+    if (e == cudaSuccess) e = e1;
     return from_cuda(e);
 }

@@ -226,6 +226,14 @@ vktError get_context(Ctx* ctx);
 void count_launches(unsigned n);
 void uncount_launches(unsigned n);   // launches that were captured into a graph, not run
 vktError from_cuda(cudaError_t e);
+// Stream-ordered scratch of a call on ctx.stream, freed with cudaFreeAsync on the same stream.
+// It comes from a pool of the library's own (one per device) that keeps up to
+// SCRATCH_KEEP_BYTES when a stream is synchronised: the default pool keeps nothing, so every
+// call after a synchronisation mapped its scratch anew (a 256^3 CLAHE-3D call alone: 293 us,
+// 76 us among others).  What is over that goes back to the driver at the next synchronisation.
+// The pool orders reuse between streams and threads itself.
+constexpr uint64_t SCRATCH_KEEP_BYTES = 64ull << 20;
+vktError scratch_alloc(void** p, size_t bytes, const Ctx& ctx);
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link).
 bool encode_tensor_map_3d(void* map /* CUtensorMap* */, int fmt, const void* base, int nx,
                           int ny, int nz, int boxx, int boxy, int boxz);

@@ -29,6 +29,7 @@ constexpr int MAX_DEVICES = 64;
 std::mutex g_mutex;
 unsigned* g_status[MAX_DEVICES] = {};
 int g_sms[MAX_DEVICES] = {};
+cudaMemPool_t g_pool[MAX_DEVICES] = {};
 // for prepare_kernel: (device, kernel, dynamic shared memory) -> resident CTAs per SM, and
 // (device, kernel) -> the largest dynamic shared memory limit set so far (the limit is never
 // lowered: a smaller setting would refuse a later launch that needs the larger one)
@@ -166,6 +167,34 @@ vktError get_context(Ctx* ctx)
     ctx->stream = static_cast<cudaStream_t>(t_policy.stream);
     ctx->debug = t_policy.debug;
     return VKT_NO_ERROR;
+}
+
+vktError scratch_alloc(void** p, size_t bytes, const Ctx& ctx)
+{
+    // (a captured allocation belongs to the graph, whatever pool it names)
+    if (stream_capturing(ctx.stream)) return from_cuda(cudaMallocAsync(p, bytes, ctx.stream));
+    cudaMemPool_t pool = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_mutex);
+        if (!g_pool[ctx.device]) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = ctx.device;
+            cudaMemPool_t made = nullptr;
+            cudaError_t e = cudaMemPoolCreate(&made, &props);
+            if (e != cudaSuccess) return from_cuda(e);
+            uint64_t keep = SCRATCH_KEEP_BYTES;
+            e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e != cudaSuccess) {
+                cudaMemPoolDestroy(made);
+                return from_cuda(e);
+            }
+            g_pool[ctx.device] = made;
+        }
+        pool = g_pool[ctx.device];
+    }
+    return from_cuda(cudaMallocFromPoolAsync(p, bytes, pool, ctx.stream));
 }
 
 vktError prepare_kernel(const Ctx& ctx, const void* kern, int threads, size_t smem, int* per_sm)
@@ -1031,13 +1060,12 @@ vktError vktApplyFilterBackwardSV(vktStructuredVolume gradSrc, float* gradWeight
         // per-CTA partial sums live in stream-ordered scratch for the duration of the call
         const size_t cap = weight_grad_scratch_floats(nx, ny, nz, k);
         float* partials = nullptr;
-        cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&partials), cap * sizeof(float),
-                                        ctx.stream);
-        if (e != cudaSuccess) return from_cuda(e);
+        err = scratch_alloc(reinterpret_cast<void**>(&partials), cap * sizeof(float), ctx);
+        if (err != VKT_NO_ERROR) return err;
         err = launch_weight_grad(static_cast<const float*>(src->data),
                                  static_cast<const float*>(gradDst->data), nx, ny, nz, k, partials,
                                  cap, gradWeights, ctx);
-        e = cudaFreeAsync(partials, ctx.stream);
+        const cudaError_t e = cudaFreeAsync(partials, ctx.stream);
         if (err == VKT_NO_ERROR && e != cudaSuccess) err = from_cuda(e);
     }
     return err;
@@ -1135,9 +1163,8 @@ vktError vktApplyFilterBackwardBatchSV(int32_t n, vktStructuredVolume* gradSrcs,
         const size_t per = weight_grad_scratch_floats(nx, ny, nz, k, 1);
         const size_t cap = one ? weight_grad_scratch_floats(nx, ny, nz, k, n) : per * n;
         float* partials = nullptr;
-        cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&partials), cap * sizeof(float),
-                                        ctx.stream);
-        if (e != cudaSuccess) return from_cuda(e);
+        err = scratch_alloc(reinterpret_cast<void**>(&partials), cap * sizeof(float), ctx);
+        if (err != VKT_NO_ERROR) return err;
         if (one) {
             err = launch_weight_grad(static_cast<const float*>(srcs[0]->data),
                                      static_cast<const float*>(gradDsts[0]->data), nx, ny, nz, k,
@@ -1151,7 +1178,7 @@ vktError vktApplyFilterBackwardBatchSV(int32_t n, vktStructuredVolume* gradSrcs,
                 err = reduce_weight_grad(partials, per * n / (static_cast<size_t>(k) * k * k), k,
                                          gradWeights, ctx);
         }
-        e = cudaFreeAsync(partials, ctx.stream);
+        const cudaError_t e = cudaFreeAsync(partials, ctx.stream);
         if (err == VKT_NO_ERROR && e != cudaSuccess) err = from_cuda(e);
     }
     return err;
