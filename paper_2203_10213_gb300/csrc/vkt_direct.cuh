@@ -36,6 +36,15 @@
 // plane of its z-march sets the pair to the product and its rounding error (dot2_first_exact),
 // which is what the addition to (0, 0) gives, so no slot is reset.  One output row per thread
 // keeps the 2 x k x RX accumulators in registers.
+//
+// Listed modes (integer sources into integer codes that FP32 could flip): the same codes at
+// nearly the price of FP32.  A voxel is evaluated in FP32 from centred codes, the value
+// mapping folded into the weights (M_LIST), or as a pair H + L of an exact high and a small
+// low part (M_PAIR, the weights split as in vkt_sep_split.cuh: two FMAs per tap); the host
+// bounds the error of either (make_list_plan), and a voxel nearer than the bound to a rounding
+// tie is put on a list in shared memory and evaluated again with the Dot2 sequence, a thread
+// per voxel.  256^3 uint8 -> uint8, k = 5 random weights: 796 us by Dot2, 116 us listed (the FMAs
+// alone 57 us at the rate a register-only loop reaches; about 1 voxel in 400 is listed).
 #pragma once
 
 #include <algorithm>
@@ -43,10 +52,16 @@
 #include <type_traits>
 
 #include "vkt_internal.h"
+#include "vkt_list_plan.h"
 #include "vkt_tile.cuh"
+#include "vkt_window.cuh"
 
 namespace vkt {
 namespace dir {
+
+// how a destination voxel is accumulated
+constexpr int M_PLAIN = 0, M_DOT2 = 1, M_LIST = 2, M_PAIR = 3;
+constexpr int LIST_AT = 512;     // listed voxels that are worked off once there are as many
 
 constexpr int NT = 256;          // threads per CTA, 16 x 16
 constexpr int BX = 16, BY = 16;
@@ -56,6 +71,20 @@ template <int K>
 struct DenseW {
     float w[K * K * K];
 };
+
+// the weights of the listed modes: those of the FMAs (w, and l in M_PAIR), the filter's own g
+// and the mapping for the listed voxels; a code is whole + frac + H + L, and tie is 1/2 less the
+// bound of its error
+template <int K, bool PAIR>
+struct ListW {
+    float w[K * K * K];
+    float l[PAIR ? K * K * K : 1];
+    float g[K * K * K];
+    float whole, frac, tie;
+    int exact;                   // sums are exact: a tie is a tie, and goes to the even code
+};
+template <int K, int MODE>
+using WeightsOf = std::conditional_t<(MODE >= M_LIST), ListW<K, MODE == M_PAIR>, DenseW<K>>;
 
 struct DirectArgs {
     const void* src;
@@ -78,10 +107,11 @@ struct DirectArgs {
 
 // SHAPE 1: one output row per thread (64 x 16 tiles) for the plain k <= 3 kernels of
 // volumes too small to give every SM a CTA (64^3: 4 tiles per plane instead of 1)
-template <int K, bool COMP = false, int SHAPE = 0>
+template <int K, int MODE = M_PLAIN, int SHAPE = 0>
 struct DirectCfg {
-    static constexpr int RX = (K == 9 || (COMP && K >= 7)) ? 2 : 4;
-    static constexpr int RY = (COMP || SHAPE == 1) ? 1 : ((K <= 3) ? 4 : 2);
+    static constexpr bool COMP = MODE == M_DOT2 || MODE == M_PAIR;   // two accumulators per output
+    static constexpr int RX = (K == 9 || (MODE == M_DOT2 && K >= 7)) ? 2 : 4;
+    static constexpr int RY = (MODE == M_PAIR && K <= 3) ? 2 : (COMP || SHAPE == 1) ? 1 : ((K <= 3) ? 4 : 2);
     static constexpr bool ROT = K >= 5;
     // PAIR: the x taps run as packed two-lane FMAs over neighbouring outputs (x, x+1),
     // which halves the FMA instructions of a kernel whose time is instruction issue
@@ -90,12 +120,15 @@ struct DirectCfg {
     using Geo = Brick<K, TX, TY>;
 };
 
-template <int K, bool COMP = false, int SHAPE = 0>
+template <int K, int MODE = M_PLAIN, int SHAPE = 0>
 __host__ __device__ constexpr size_t direct_smem_bytes(int sfmt, bool rows)
 {
-    using Geo = typename DirectCfg<K, COMP, SHAPE>::Geo;
+    using Geo = typename DirectCfg<K, MODE, SHAPE>::Geo;
     return 128 + static_cast<size_t>(STAGES) * Geo::stage_bytes(sfmt, rows) +
-           2 * static_cast<size_t>(Geo::FH) * Geo::FP * sizeof(float);
+           2 * static_cast<size_t>(Geo::FH) * Geo::FP * sizeof(float) +
+           (MODE >= M_LIST ? (LIST_AT + DirectCfg<K, MODE, SHAPE>::TX * DirectCfg<K, MODE, SHAPE>::TY + 4) *
+                                 sizeof(uint32_t)
+                           : 0);
 }
 
 // SF/DF: source and destination formats fixed at compile time (-1: read from the arguments);
@@ -103,16 +136,59 @@ __host__ __device__ constexpr size_t direct_smem_bytes(int sfmt, bool rows)
 // so code for unused ways of loading costs instruction cache): 0 = from the arguments
 // (tensor map, row copies or plain loads), 1 = tensor map, 2 = row copies
 constexpr int LM_ANY = 0, LM_TMA = 1, LM_ROWS = 2;
+// the Dot2 code of voxel (x, y, z): the taps in the order and with the operations of the
+// compensated kernel.  The voxels of a plane are loaded before its chain of K^2 steps, which
+// hides all but one load latency per plane.
+template <int K>
+__device__ __noinline__ unsigned dot2_voxel(const void* src, int sfmt, int nx, int ny, int nz, int x,
+                                            int y, int z, const float* g, float a0, float a0lo,
+                                            float a1, float a1lo, float qmax)
+{
+    constexpr int R = (K - 1) / 2, B = K <= 7 ? K : 3;   // rows loaded together
+    float s = 0.f, e = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < K; ++c) {
+        const int64_t pl = static_cast<int64_t>(clampi(z + c - R, 0, nz - 1)) * ny;
+#pragma unroll 1
+        for (int b0 = 0; b0 < K; b0 += B) {
+            float v[B][K];
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const int64_t row = (pl + clampi(y + b0 + b - R, 0, ny - 1)) * nx;
+#pragma unroll
+                for (int a = 0; a < K; ++a) {
+                    const int64_t i = row + clampi(x + a - R, 0, nx - 1);
+                    v[b][a] = sfmt == FMT_U16
+                                  ? static_cast<float>(__ldg(static_cast<const uint16_t*>(src) + i))
+                                  : static_cast<float>(__ldg(static_cast<const unsigned char*>(src) + i));
+                }
+            }
+            const float* w = g + (c * K + b0) * K;
+#pragma unroll
+            for (int b = 0; b < B; ++b)
+#pragma unroll
+                for (int a = 0; a < K; ++a) {
+                    if (c == 0 && b0 == 0 && b == 0 && a == 0)
+                        dot2_first_exact(w[0], v[0][0], s, e);
+                    else
+                        dot2_exact(w[b * K + a], v[b][a], s, e);
+                }
+        }
+    }
+    return comp_code(s, e, a0, a0lo, a1, a1lo, qmax);
+}
+
 // ROI: the forward stores are bounded by the arguments' region fields; otherwise by the
-// volume (known at compile time to start at column 0).  COMP: compensated accumulation
+// volume (known at compile time to start at column 0).  MODE: see above; other than M_PLAIN
 // into an integer destination (forward only).
 template <int K, bool ADJ, int SF = -1, int DF = -1, int LM = LM_ANY, bool ROI = false,
-          bool COMP = false, int SHAPE = 0>
-__global__ void __launch_bounds__(NT)
-    k_direct(const __grid_constant__ CUtensorMap tmap, const DirectArgs p, const DenseW<K> W)
+          int MODE = M_PLAIN, int SHAPE = 0>
+__device__ __forceinline__ void direct_body(const CUtensorMap& tmap, const DirectArgs& p,
+                                            const WeightsOf<K, MODE>& W)
 {
-    static_assert(!(COMP && ADJ), "the adjoint writes float32");
-    using Cfg = DirectCfg<K, COMP, SHAPE>;
+    static_assert(!(MODE != M_PLAIN && ADJ), "the adjoint writes float32");
+    constexpr bool COMP = DirectCfg<K, MODE, SHAPE>::COMP, LISTED = MODE >= M_LIST;
+    using Cfg = DirectCfg<K, MODE, SHAPE>;
     using Geo = typename Cfg::Geo;
     constexpr int R = Geo::R, RX = Cfg::RX, RY = Cfg::RY;
     constexpr int FH = Geo::FH, FP = Geo::FP;
@@ -127,9 +203,11 @@ __global__ void __launch_bounds__(NT)
     const uint32_t txb = Geo::raw_tx(sfmt);
     unsigned char* raw = smem + 128;
     float* F = reinterpret_cast<float*>(raw + STAGES * rawb);
+    uint32_t* list = reinterpret_cast<uint32_t*>(F + 2 * FH * FP);
+    volatile uint32_t* count = list + (LISTED ? LIST_AT + Cfg::TX * Cfg::TY : 0);
     // a launch whose shared memory was sized for another tile shape records the mismatch
     // and does nothing (instead of running past the end of its shared memory)
-    if (dynamic_smem_bytes() < direct_smem_bytes<K, COMP, SHAPE>(sfmt, rows)) {
+    if (dynamic_smem_bytes() < direct_smem_bytes<K, MODE, SHAPE>(sfmt, rows)) {
         grid_dependency_wait();
         if (threadIdx.x == 0) atomicOr(p.status, STATUS_CONFIG);
         return;
@@ -153,6 +231,7 @@ __global__ void __launch_bounds__(NT)
         for (int s = 0; s < STAGES; ++s) mbar_init(&bars[s], 1);
         fence_mbar_init();
         if (LM != LM_ROWS && p.use_tma) prefetch_tensor_map(&tmap);
+        if constexpr (LISTED) *count = 0;
     }
     __syncthreads();
     // set-up done: wait for the previous kernel on the stream (programmatic launch), let
@@ -213,6 +292,26 @@ __global__ void __launch_bounds__(NT)
     const int yend = ROI ? p.sy1 : p.ny;
     bool failed = false;
 
+    // evaluates the listed voxels again (all threads; the caller synchronises around it)
+    auto work_off = [&]() {
+        if constexpr (LISTED) {
+            const uint32_t n = *count;
+            for (uint32_t i = tid; i < n; i += NT) {
+                const uint32_t e = list[i];
+                const int x = x0 + static_cast<int>(e % Cfg::TX);
+                const int y = y0 + static_cast<int>(e / Cfg::TX % Cfg::TY);
+                const int z = zc0 + static_cast<int>(e / (Cfg::TX * Cfg::TY));
+                const unsigned code = dot2_voxel<K>(src, sfmt, p.nx, p.ny, p.nz, x, y, z, W.g, p.a0,
+                                                    p.a0lo, p.a1, p.a1lo, p.qmax);
+                const int64_t idx = (static_cast<int64_t>(z) * p.ny + y) * p.nx + x;
+                if (dfmt == FMT_U16)
+                    static_cast<uint16_t*>(dst)[idx] = static_cast<uint16_t>(code);
+                else
+                    static_cast<unsigned char*>(dst)[idx] = static_cast<unsigned char>(code);
+            }
+        }
+    };
+
     // One input plane: fetch, convert, multiply into the K output planes, retire one.
     auto plane = [&](const int it, const int u) {
         const int s = it % STAGES;
@@ -232,15 +331,28 @@ __global__ void __launch_bounds__(NT)
                     const uint32_t zterm =
                         static_cast<uint32_t>(clampi(pfirst + it, 0, p.nz - 1)) *
                         static_cast<uint32_t>(p.ny) * static_cast<uint32_t>(p.nx);
-                    plan.convert_rows(rs, sfmt, Fb, tid, p.nx, p.ny, x0, y0, zterm);
+                    plan.template convert_rows<LISTED>(rs, sfmt, Fb, tid, p.nx, p.ny, x0, y0, zterm);
                 } else {
-                    plan.convert(rs, sfmt, Fb, tid);
+                    plan.template convert<LISTED>(rs, sfmt, Fb, tid);
                 }
             } else {
                 plan.convert(rs, sfmt, Fb, tid);
             }
         }
-        if (__syncthreads_or(!ok)) {
+        if constexpr (LISTED) {
+            // every voxel of the planes before is listed: whoever lists the last of LIST_AT voxels
+            // sees the full count here
+            if (__syncthreads_or(!ok || *count >= LIST_AT)) {
+                if (__syncthreads_or(!ok)) {
+                    failed = true;
+                    return;
+                }
+                work_off();
+                __syncthreads();
+                if (tid == 0) *count = 0;
+                __syncthreads();
+            }
+        } else if (__syncthreads_or(!ok)) {
             failed = true;
             return;
         }
@@ -299,7 +411,17 @@ __global__ void __launch_bounds__(NT)
 #pragma unroll
                 for (int c = 0; c < K; ++c) {
                     const int sl = Cfg::ROT ? (K - 1 - c) : (((u - c + R) % K + K) % K);
-                    if constexpr (COMP) {
+                    if constexpr (MODE == M_PAIR) {
+#pragma unroll
+                        for (int x = 0; x < RX; ++x)
+#pragma unroll
+                            for (int a = 0; a < K; ++a) {
+                                const int t = (c * K + b) * K + a;
+                                float &H = cs[sl][i][x], &L = cc[sl][i][x];
+                                H = t == 0 ? __fmul_rn(W.w[t], win[x + a]) : __fmaf_rn(W.w[t], win[x + a], H);
+                                L = t == 0 ? __fmul_rn(W.l[t], win[x + a]) : __fmaf_rn(W.l[t], win[x + a], L);
+                            }
+                    } else if constexpr (COMP) {
 #pragma unroll
                         for (int x = 0; x < RX; ++x)
 #pragma unroll
@@ -341,7 +463,55 @@ __global__ void __launch_bounds__(NT)
         }
         // output plane it - 2R + zc0 is complete
         const int sl0 = Cfg::ROT ? 0 : (((u - R) % K + K) % K);
+        if constexpr (LISTED) {
+            if (it >= 2 * R) {
+                const int oz = pfirst + it - R;
+#pragma unroll
+                for (int i = 0; i < RY; ++i) {
+                    const int oy = y0 + ty * RY + i;
+                    if (oy < yend && nvalid > 0) {
+                        unsigned code[RX];
+                        float rest[RX], most = 0.f;
+#pragma unroll
+                        for (int x = 0; x < RX; ++x) {
+                            float H, L = W.frac;
+                            if constexpr (MODE == M_PAIR) {
+                                H = cs[sl0][i][x];
+                                L = __fadd_rn(cc[sl0][i][x], W.frac);
+                            } else {
+                                H = lane(sl0, i, x);
+                            }
+                            // the nearest integer of H, then of what is left and L
+                            const float m0 = __fsub_rn(__fadd_rn(H, 12582912.f), 12582912.f);
+                            const float s2 = __fadd_rn(__fsub_rn(H, m0), L);
+                            const float m1 = __fsub_rn(__fadd_rn(s2, 12582912.f), 12582912.f);
+                            const float r = __fsub_rn(s2, m1);
+                            rest[x] = fabsf(r);
+                            most = fmaxf(most, rest[x]);
+                            float qf = __fadd_rn(m0, __fadd_rn(m1, W.whole));
+                            // (qf is an integer below 2^22: its last bit, in 1.5 * 2^23 + qf)
+                            if (MODE == M_LIST && W.exact && rest[x] == 0.5f &&
+                                (__float_as_uint(__fadd_rn(qf, 12582912.f)) & 1u))
+                                qf = __fadd_rn(qf, r > 0.f ? 1.f : -1.f);
+                            // an integer in [0, 2^16) added to 2^23 stands in the low bits
+                            code[x] = __float_as_uint(fminf(fmaxf(qf, 0.f), p.qmax) + 8388608.f) & 0xFFFFu;
+                        }
+                        const int64_t idx = (static_cast<int64_t>(oz) * p.ny + oy) * p.nx + ox;
+                        store_codes<RX>(dst, dfmt, idx, first, nvalid, code);
+                        if (most >= W.tie) {
+                            const uint32_t at = (static_cast<uint32_t>(oz - zc0) * Cfg::TY + ty * RY + i) * Cfg::TX +
+                                                tx * RX;
+#pragma unroll
+                            for (int x = 0; x < RX; ++x)
+                                if (rest[x] >= W.tie && x >= first && x < nvalid)
+                                    list[atomicAdd(const_cast<uint32_t*>(count), 1u)] = at + x;
+                        }
+                    }
+                }
+            }
+        }
         if constexpr (COMP) {
+            if constexpr (MODE == M_DOT2)
             if (it >= 2 * R) {
                 const int oz = pfirst + it - R;
 #pragma unroll
@@ -375,7 +545,7 @@ __global__ void __launch_bounds__(NT)
             }
             return;
         }
-        if (it >= 2 * R) {
+        if (!LISTED && it >= 2 * R) {
             const int oz = pfirst + it - R;
 #pragma unroll
             for (int i = 0; i < RY; ++i) {
@@ -426,7 +596,39 @@ __global__ void __launch_bounds__(NT)
                 if (it != 0 || !p.withhold_first) mbar_wait(&bars[it % STAGES], (it / STAGES) & 1);
         }
         __syncthreads();
+    } else if constexpr (LISTED) {
+        __syncthreads();   // every voxel is listed and its first code stored
+        work_off();
     }
+}
+
+template <int K, bool ADJ, int SF = -1, int DF = -1, int LM = LM_ANY, bool ROI = false,
+          int MODE = M_PLAIN, int SHAPE = 0>
+__global__ void __launch_bounds__(NT)
+    k_direct(const __grid_constant__ CUtensorMap tmap, const DirectArgs p, const DenseW<K> W)
+{
+    direct_body<K, ADJ, SF, DF, LM, ROI, MODE, SHAPE>(tmap, p, W);
+}
+
+// The listed modes: their weights are also read by index (dot2_voxel), so they stay where the
+// launch put them (in the other kernels that costs the compiler its register allocation: k = 3
+// on 512^3 194 -> 206 us), and two CTAs fit an SM (the call would take up to 255 registers).
+template <int K, int LM, bool ROI, int MODE, int SHAPE>
+__global__ void __launch_bounds__(NT, K <= 7 ? 2 : 1)
+    k_direct_listed(const __grid_constant__ CUtensorMap tmap, const DirectArgs p,
+                    const __grid_constant__ WeightsOf<K, MODE> W)
+{
+    direct_body<K, false, -1, -1, LM, ROI, MODE, SHAPE>(tmap, p, W);
+}
+
+// the kernel of one mode with the formats read from the arguments
+template <int K, bool ADJ, int LM, bool ROI, int MODE, int SHAPE>
+constexpr auto kernel_of()
+{
+    if constexpr (MODE >= M_LIST)
+        return &k_direct_listed<K, LM, ROI, MODE, SHAPE>;
+    else
+        return &k_direct<K, ADJ, -1, -1, LM, ROI, MODE, SHAPE>;
 }
 
 // The adjoint's shell: the positions j' of [-r, n+r)^3 outside [0, n)^3, each of whose
@@ -595,12 +797,13 @@ inline bool direct_small(const Job& job, int sms)
 }
 
 // One launch of the direct kernel over the job's region (forward) or over the padded
-// domain (adjoint); COMP: compensated accumulation into an integer destination.
-template <int K, bool ADJ, bool COMP = false, int SHAPE = 0>
-vktError launch_k(const Job& job, const float* w, const Ctx& ctx)
+// domain (adjoint); MODE: how an integer destination is accumulated.
+// plan: the weights of the listed modes.
+template <int K, bool ADJ, int MODE = M_PLAIN, int SHAPE = 0>
+vktError launch_k(const Job& job, const float* w, const Ctx& ctx, const ListPlan* plan = nullptr)
 {
-    static_assert(!(COMP && ADJ), "the adjoint writes float32");
-    using Cfg = DirectCfg<K, COMP, SHAPE>;
+    static_assert(!(MODE != M_PLAIN && ADJ), "the adjoint writes float32");
+    using Cfg = DirectCfg<K, MODE, SHAPE>;
     using Geo = typename Cfg::Geo;
     constexpr int R = Geo::R;
     DirectArgs a;
@@ -642,9 +845,21 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx)
         a.sx1 = rx1;
         a.sy1 = ry1;
     }
-    DenseW<K> W;
+    WeightsOf<K, MODE> W;
     const int kk = K * K * K;
-    for (int i = 0; i < kk; ++i) W.w[i] = ADJ ? w[kk - 1 - i] : w[i];   // adjoint: w[-d]
+    if constexpr (MODE >= M_LIST) {
+        for (int i = 0; i < kk; ++i) {
+            W.w[i] = plan->w[i];
+            if constexpr (MODE == M_PAIR) W.l[i] = plan->l[i];
+            W.g[i] = w[i];
+        }
+        W.whole = plan->whole;
+        W.frac = plan->frac;
+        W.tie = plan->tie;
+        W.exact = plan->exact;
+    } else {
+        for (int i = 0; i < kk; ++i) W.w[i] = ADJ ? w[kk - 1 - i] : w[i];   // adjoint: w[-d]
+    }
 
     const int gx = (a.ex + Cfg::TX - 1) / Cfg::TX;
     const int gy = (a.ey + Cfg::TY - 1) / Cfg::TY;
@@ -672,34 +887,34 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx)
                  ? 1
                  : 0;
 
-    const size_t smem = direct_smem_bytes<K, COMP, SHAPE>(job.sfmt, a.rows != 0);
+    const size_t smem = direct_smem_bytes<K, MODE, SHAPE>(job.sfmt, a.rows != 0);
     // the common float32 destinations get kernels with their formats compiled in
     // tensor-map jobs get kernels without the other ways of loading, and so do row-copy
     // jobs of the compiled-in formats; plain-load jobs take the run-time variant
-    auto kern = a.use_tma ? k_direct<K, ADJ, -1, -1, LM_TMA, false, COMP, SHAPE>
-                          : k_direct<K, ADJ, -1, -1, LM_ANY, false, COMP, SHAPE>;
+    auto kern = a.use_tma ? kernel_of<K, ADJ, LM_TMA, false, MODE, SHAPE>()
+                          : kernel_of<K, ADJ, LM_ANY, false, MODE, SHAPE>();
     if constexpr (!ADJ) {
-        if (job.roi) kern = k_direct<K, ADJ, -1, -1, LM_ANY, true, COMP, SHAPE>;   // reads the region fields
+        if (job.roi) kern = kernel_of<K, ADJ, LM_ANY, true, MODE, SHAPE>();   // reads the region fields
     }
-    if constexpr (!ADJ && !COMP && K >= 3 && K <= 5) {
+    if constexpr (!ADJ && MODE == M_PLAIN && K >= 3 && K <= 5) {
         // region tensor-map jobs of the common float32 destinations: formats compiled in
         if (job.roi && a.use_tma && job.dfmt == FMT_F32 && job.sfmt == FMT_U8)
-            kern = k_direct<K, ADJ, FMT_U8, FMT_F32, LM_TMA, true, false, SHAPE>;
+            kern = k_direct<K, ADJ, FMT_U8, FMT_F32, LM_TMA, true, M_PLAIN, SHAPE>;
         if (job.roi && a.use_tma && job.dfmt == FMT_F32 && job.sfmt == FMT_F32)
-            kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_TMA, true, false, SHAPE>;
+            kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_TMA, true, M_PLAIN, SHAPE>;
     }
     if constexpr (ADJ && K >= 3 && K <= 5) {
         // the adjoint reads and writes float32: formats compiled in for tensor-map jobs
-        if (a.use_tma) kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_TMA, false, false, SHAPE>;
+        if (a.use_tma) kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_TMA, false, M_PLAIN, SHAPE>;
     }
-    if constexpr (!ADJ && !COMP && K >= 3 && K <= 5) {
+    if constexpr (!ADJ && MODE == M_PLAIN && K >= 3 && K <= 5) {
         if (!job.roi && job.dfmt == FMT_F32 && job.sfmt == FMT_U8) {
-            if (a.use_tma) kern = k_direct<K, ADJ, FMT_U8, FMT_F32, LM_TMA, false, false, SHAPE>;
-            else if (a.rows) kern = k_direct<K, ADJ, FMT_U8, FMT_F32, LM_ROWS, false, false, SHAPE>;
+            if (a.use_tma) kern = k_direct<K, ADJ, FMT_U8, FMT_F32, LM_TMA, false, M_PLAIN, SHAPE>;
+            else if (a.rows) kern = k_direct<K, ADJ, FMT_U8, FMT_F32, LM_ROWS, false, M_PLAIN, SHAPE>;
         }
         if (!job.roi && job.dfmt == FMT_F32 && job.sfmt == FMT_F32) {
-            if (a.use_tma) kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_TMA, false, false, SHAPE>;
-            else if (a.rows) kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_ROWS, false, false, SHAPE>;
+            if (a.use_tma) kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_TMA, false, M_PLAIN, SHAPE>;
+            else if (a.rows) kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_ROWS, false, M_PLAIN, SHAPE>;
         }
     }
     int per_sm = 1;
@@ -714,7 +929,7 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx)
     if (a.use_tma && per_launch < nvol && !encode(job.src, per_launch)) return VKT_ERROR_CUDA;
     if (ctx.debug & VKT_DEBUG_LOG)
         fprintf(stderr, "[vkt] direct%s k=%d grid=(%d,%d,%d) zchunk=%d smem=%zu tma=%d rows=%d withhold=%d\n",
-                ADJ ? "-adjoint" : (COMP ? "-compensated" : ""), K, gx, gy, gz, a.zchunk, smem,
+                ADJ ? "-adjoint" : (MODE == M_DOT2 ? "-compensated" : MODE == M_LIST ? "-listed" : MODE == M_PAIR ? "-listed-pair" : ""), K, gx, gy, gz, a.zchunk, smem,
                 a.use_tma, a.rows, a.withhold_first);
     const DirectArgs a0 = a;
     for (int v0 = 0; v0 < nvol; v0 += per_launch) {

@@ -179,6 +179,10 @@ vktError prepare_kernel(const Ctx& ctx, const void* kern, int threads, size_t sm
 // the compensated kernels when job.comp is set (launch_direct_comp).
 vktError launch_direct(const Job& job, const float* w, int k, const Ctx& ctx);
 vktError launch_direct_comp(const Job& job, const float* w, int k, const Ctx& ctx);
+// The listed modes of the compensated direct kernel, where they suit the job (*taken).
+struct ListPlan;
+vktError launch_direct_listed(const Job& job, const float* w, int k, const Ctx& ctx, bool* taken);
+vktError launch_direct_pair(const Job& job, const float* w, int k, const Ctx& ctx, const ListPlan& plan);
 // dL/dsrc of the clamped correlation (float32 gy in job.src, gx in job.dst): every voxel of
 // gx is written (the main launch), then the shell outside the volume is added to the face
 // voxels (a second, small launch).

@@ -6,6 +6,7 @@
 #include <cmath>
 
 #include "vkt_internal.h"
+#include "vkt_list_plan.h"
 
 namespace vkt {
 
@@ -38,7 +39,7 @@ inline bool weights(const double* g, int k, double v, double b, float* hi, float
 // Fills `p` for the vectors g[0..2] of size k over a source of integer format sfmt (0: uint8,
 // 1: uint16) and the uncentred code mapping a0 + a1 * sum (a0 = a0h + a0l, ...).  False if the
 // evaluation does not suit the filter: weights that are not finite, results far outside the
-// codes, or an error bound over 1/100 of a code (more than 1 in 50 voxels would be evaluated
+// codes, flat regions on ties, or an error bound over 1/100 of a code (more than 1 in 50 voxels would be evaluated
 // twice).
 inline bool make_split_plan(SplitPlan& p, int k, const float* const g[3], int sfmt, float a0h,
                             float a0l, float a1h, float a1l)
@@ -109,7 +110,8 @@ inline bool make_split_plan(SplitPlan& p, int k, const float* const g[3], int sf
     // itself may be off (errors of second order, below 1e-7 of a 16-bit code)
     const double e = err + 3.0 * u * (bl + 2.0) + 1e-6 * std::max(1.0, reach / 65536.0);
     p.tie = static_cast<float>(0.5 - e * 1.0001) * (1.f - 1.2e-7f);
-    return e < 0.01;
+    const double slope = sum[0] * sum[1] * sum[2];
+    return e < 0.01 && !flat_field_ties(a0 - b0 * slope, slope, sfmt, e);
 }
 
 }  // namespace vkt

@@ -345,10 +345,13 @@ struct ConvPlan {
         }
     }
 
-    // raw tile -> float tile (pitch FP), every element mapped to its clamped voxel
+    // raw tile -> float tile (pitch FP), every element mapped to its clamped voxel (CENTRE: minus
+    // half the range of an integer format)
+    template <bool CENTRE = false>
     __device__ __forceinline__ void convert(const unsigned char* raw, int fmt, float* F,
                                             int tid) const
     {
+        const float sub = fmt == FMT_U8 ? 128.f : 32768.f;
 #pragma unroll
         for (int n = 0; n < NG; ++n) {
             const int gi = tid + n * NT;
@@ -363,16 +366,19 @@ struct ConvPlan {
             } else {
                 v = make_float4(raw[off[n][0]], raw[off[n][1]], raw[off[n][2]], raw[off[n][3]]);
             }
+            if constexpr (CENTRE) v = make_float4(v.x - sub, v.y - sub, v.z - sub, v.w - sub);
             reinterpret_cast<float4*>(F)[gi] = v;
         }
     }
 
     // the same for a stage filled by issue_rows (clamped conversion only): each row's
     // elements sit row_shift_elems() further in; zterm = clamp(z) * ny * nx (mod 2^32)
+    template <bool CENTRE = false>
     __device__ __forceinline__ void convert_rows(const unsigned char* raw, int fmt, float* F,
                                                  int tid, int nx, int ny, int x0, int y0,
                                                  uint32_t zterm) const
     {
+        const float sub = fmt == FMT_U8 ? 128.f : 32768.f;
         static_assert(CLAMP, "row-copied stages hold only rows inside the volume");
         const int xa = fmt_xalign(fmt);
 #pragma unroll
@@ -393,6 +399,7 @@ struct ConvPlan {
                 const unsigned char* r = raw + m;
                 v = make_float4(r[off[n][0]], r[off[n][1]], r[off[n][2]], r[off[n][3]]);
             }
+            if constexpr (CENTRE) v = make_float4(v.x - sub, v.y - sub, v.z - sub, v.w - sub);
             reinterpret_cast<float4*>(F)[gi] = v;
         }
     }
