@@ -98,7 +98,7 @@ struct DirectArgs {
     int gzv;               // z chunks per volume: blockIdx.z = volume * gzv + chunk
     int64_t vs_src, vs_dst;   // voxels from one volume of the batch to the next
     int use_tma;
-    int rows;              // no tensor map: stages filled by per-row bulk copies (forward only)
+    int rows;              // no tensor map: stages filled by row copies (forward only)
     int withhold_first;    // fault injection: the first plane's TMA load is never issued
     float a0, a1, qmax;
     float a0lo, a1lo;      // compensated mode: low halves of a0, a1 (double-float pairs)
@@ -879,8 +879,8 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx, const ListPlan
     // encoded for the whole batch first and re-encoded per launch once gz is known
     a.use_tma = encode(job.src, std::min(nvol, 65535)) ? 1 : 0;
     if (!a.use_tma) memset(&map, 0, sizeof(map));
-    // rows that no tensor map can describe are still fetched asynchronously, one bulk copy
-    // per row, when every volume starts on a 16-byte boundary (forward only: the adjoint
+    // rows that no tensor map can describe are still fetched asynchronously, as 16-byte blocks,
+    // when every volume starts on a 16-byte boundary (forward only: the adjoint
     // needs the zero extension a tensor map or the plain loads give)
     a.rows = (!ADJ && !a.use_tma && reinterpret_cast<uintptr_t>(job.src) % 16 == 0 &&
               (job.vs_src * es) % 16 == 0)

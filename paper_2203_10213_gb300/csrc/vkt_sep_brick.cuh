@@ -14,6 +14,7 @@
 
 #include "vkt_internal.h"
 #include "vkt_tile.cuh"
+#include "vkt_window.cuh"
 
 namespace vkt {
 namespace sep {
@@ -44,7 +45,7 @@ struct Job {
     int sfmt, dfmt;
     int zchunk;
     int use_tma;
-    int rows;          // no tensor map: stages filled by per-row bulk copies (issue_rows)
+    int rows;          // no tensor map: stages filled by row copies (issue_rows)
     // output region: bricks start at (ox0, oy0, oz0) and store the voxels with x in
     // [sx0, sx1), y < sy1, z < sz1 (the whole volume: set_whole_volume)
     int ox0, oy0, oz0;
@@ -72,24 +73,20 @@ struct W {
     float gx[K], gy[K], gz[K];
 };
 
-// FX: the x pass reads the raw tensor-map stage directly (converting as it loads) into one of
-// two x-pass tiles, so a plane needs one CTA barrier instead of two, no float tile, and none
-// of the float tile's shared-memory traffic (about 14 of the 30 bytes per output voxel).  For
-// float32 sources with tensor-map loads (17-21 % faster at k = 3, 5) and for uint8 sources,
-// whose window is read as three aligned 32-bit words and converted with a byte permute
-// (byte_float) instead of one byte load and one conversion per voxel (k = 5 on 512^3:
-// 0.209 -> 0.199 ms at two CTAs per SM; at three it spills)
+// FX: the x pass reads the raw stage directly (converting as it loads) into one of two x-pass
+// tiles, so a plane needs one CTA barrier instead of two, no float tile, and none of the float
+// tile's shared-memory traffic (about 14 of the 30 bytes per output voxel).  For float32
+// sources with tensor-map loads (17-21 % faster at k = 3, 5) and for integer sources, without a
+// tensor map up to k = 5 (at k = 7 a window of 10 codes at any alignment costs more than the
+// float tile: 302^3 uint8 into float32 118 against 102 us): their window is read as aligned 32-bit words and converted with a byte
+// permute (vkt_window.cuh) instead of one load and one conversion per voxel.  uint8, k = 5:
+// 512^3 into float32 0.209 -> 0.199 ms at two CTAs per SM (at three it spills), 256x256x200 into
+// uint8 49 -> 29 us, 302^3 into uint8 (row copies) 108 -> 88 us.
 template <int LM, int SF, int K>
 __host__ __device__ constexpr bool fused_x()
 {
-    return LM == LM_TMA && (SF == FMT_F32 || SF == FMT_U8);
-}
-
-// byte i (0..3) of word w as the float it codes (exact): 2^23 + code built by a byte permute,
-// minus 2^23
-__device__ __forceinline__ float byte_float(uint32_t w, int i)
-{
-    return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u + i)) - 8388608.f;
+    if (SF == FMT_F32) return LM == LM_TMA;
+    return (SF == FMT_U8 || SF == FMT_U16) && (LM == LM_TMA || K <= 5);
 }
 
 // the output tile of a brick with BXG threads along x (64 x 32 by default, 32 x 32 narrow)
@@ -102,10 +99,10 @@ template <int BXG>
 constexpr int tile_y_comp() { return (NT / BXG) * CRY; }
 
 template <int K, int NS = FSTAGES, int BXG = BX>
-__host__ __device__ constexpr size_t smem_bytes_fx(int sfmt)
+__host__ __device__ constexpr size_t smem_bytes_fx(int sfmt, bool rows = false)
 {
     using Geo = Brick<K, tile_x<BXG>(), tile_y<BXG>()>;
-    return 128 + static_cast<size_t>(NS) * Geo::stage_bytes(sfmt, false) +
+    return 128 + static_cast<size_t>(NS) * Geo::stage_bytes(sfmt, rows) +
            2 * static_cast<size_t>(Geo::FH) * tile_x<BXG>() * sizeof(float);
 }
 
@@ -118,11 +115,24 @@ __host__ __device__ constexpr size_t smem_bytes(int sfmt, bool rows = false)
            static_cast<size_t>(Geo::FH) * tile_x<BXG>() * sizeof(float);  // x-pass output
 }
 
+// row copies of a plane, by the way the kernel uses
+template <typename Geo, bool BULK, typename... A>
+__device__ __forceinline__ void copy_rows(A... a)
+{
+    if constexpr (BULK)
+        issue_rows_bulk<Geo, NT>(a...);
+    else
+        issue_rows<Geo, NT>(a...);
+}
+
+constexpr int XBAR = 9;   // the barrier of the split brick's x passes
+
 // Initialises the stage barriers (thread 0; the caller synchronises afterwards).
 __device__ __forceinline__ void init_barriers(unsigned char* smem)
 {
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem);
     for (int s = 0; s < 9; ++s) mbar_init(&bars[s], 1);   // up to 9 stages (in the 128-byte header)
+    mbar_init(&bars[XBAR], NT / 32);                      // an arrival per warp
     fence_mbar_init();
 }
 
@@ -145,7 +155,7 @@ __device__ __forceinline__ void init_barriers(unsigned char* smem)
 // arithmetic.  A persistent CTA (the batch) carries gplane from brick to brick and must use
 // the general ring, whatever NS and K are.
 template <int K, class Wt, int SF = -1, int DF = -1, int LM = LM_ANY, bool ROI = false,
-          int NS = FSTAGES, bool STATIC = false, bool ROTZ = false, int BXG = BX>
+          int NS = FSTAGES, bool STATIC = false, bool ROTZ = false, int BXG = BX, bool BULK = false>
 __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorMap* tmap, int bx,
                                       int by, int bz, unsigned char* smem, uint32_t& gplane,
                                       unsigned* status)
@@ -201,13 +211,15 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
     } else if (rows) {
         for (int s = 0; s < NS && s < nplanes; ++s) {
             const uint32_t q = g0 + s;
-            issue_rows<Geo, NT>(raw + (q % NS) * rawb, &bars[q % NS], J.src, vol_bytes,
+            copy_rows<Geo, BULK>(raw + (q % NS) * rawb, &bars[q % NS], J.src, vol_bytes,
                                 sfmt, J.nx, J.ny, J.nz, x0, y0, pfirst + s, tid);
         }
         __syncthreads();   // every thread's expect_tx precedes the single arrival
         if (tid == 0)
             for (int s = 0; s < NS && s < nplanes; ++s, ++issued) mbar_arrive(&bars[(g0 + s) % NS]);
     }
+
+    int pend = -1;   // FX: a stage refilled by row copies, to be given its arrival
 
     ConvPlan<Geo, NT> plan;
     plan.init(sfmt, J.nx, J.ny, x0, y0, tid, rows);
@@ -246,39 +258,30 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
         bool ok = true;
         if constexpr (FX) {
             float* T1b = T1 + (it & 1) * FH * TX;
-            ok = mbar_wait(&bars[s], par);
+            if (tma || rows) {
+                ok = mbar_wait(&bars[s], par);
+            } else {
+                fill_raw_plain<Geo, NT>(const_cast<unsigned char*>(rs), J.src, sfmt, J.nx, J.ny,
+                                        J.nz, x0, y0, pfirst + it, tid);
+                __syncthreads();
+            }
             // x pass straight from the raw stage: T1b[row][x] = sum_a gx[a] v(x + a - r), the
             // source voxels converted as they are loaded, clamped in x only at the volume's
             // x faces (the rows are clamped through the stage row read)
-            constexpr int RWE = TX + 2 * fmt_xalign(SF);   // raw row length in voxels
             const bool xin = x0 - R >= 0 && x0 + TX - 1 + R <= J.nx - 1;
+            const uint32_t zterm = static_cast<uint32_t>(clampi(pfirst + it, 0, J.nz - 1)) *
+                                   static_cast<uint32_t>(J.ny) * static_cast<uint32_t>(J.nx);
             if (ok) {
 #pragma unroll
                 for (int n = 0; n < (XITEMS + NT - 1) / NT; ++n) {
                     const int item = tid + n * NT;
                     if (item < XITEMS) {
                         const int row = item / XGROUPS, g = item - row * XGROUPS;
-                        const int rrow = clampi(y0 - R + row, 0, J.ny - 1) - (y0 - R);
+                        const int gy = clampi(y0 - R + row, 0, J.ny - 1);
+                        const int rrow = gy - (y0 - R);
                         float win[4 + K - 1];
-                        if constexpr (SF == FMT_U8) {
-                            const unsigned char* rp = rs + rrow * RWE;
-                            if (xin) {
-                                // the item's K + 3 bytes start at raw column 4g + xa - R
-                                // (xa = 16): the three aligned words from word g + W0 cover them
-                                constexpr int W0 = (16 - R) / 4, O = (16 - R) & 3;
-                                static_assert(O + K + 3 <= 12, "three words hold the window");
-                                const uint32_t* wp = reinterpret_cast<const uint32_t*>(rp) + g + W0;
-                                const uint32_t wd[3] = {wp[0], wp[1], wp[2]};
-#pragma unroll
-                                for (int e = 0; e < 4 + K - 1; ++e)
-                                    win[e] = byte_float(wd[(O + e) >> 2], (O + e) & 3);
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < 4 + K - 1; ++e)
-                                    win[e] = static_cast<float>(
-                                        rp[clampi(x0 + 4 * g - R + e, 0, J.nx - 1) - (x0 - xa)]);
-                            }
-                        } else {
+                        if constexpr (SF == FMT_F32) {
+                            constexpr int RWE = TX + 2 * fmt_xalign(SF);   // raw row length in voxels
                             const float* rp = reinterpret_cast<const float*>(rs) + rrow * RWE;
                             if (xin) {
 #pragma unroll
@@ -288,6 +291,25 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
                                 for (int e = 0; e < 4 + K - 1; ++e)
                                     win[e] = rp[clampi(x0 + 4 * g - R + e, 0, J.nx - 1) - (x0 - xa)];
                             }
+                        } else if constexpr (LM == LM_TMA) {
+                            const unsigned char* rp = rs + rrow * Geo::raw_w(SF) * fmt_bytes(SF);
+                            if (xin) {
+                                window<K, SF, true, false>(rp, 4 * g + fmt_xalign(SF) - R, 0u, win);
+                            } else {
+#pragma unroll
+                                for (int e = 0; e < 4 + K - 1; ++e) {
+                                    const int at = clampi(x0 + 4 * g - R + e, 0, J.nx - 1) - (x0 - xa);
+                                    win[e] = SF == FMT_U8
+                                                 ? static_cast<float>(rp[at])
+                                                 : static_cast<float>(reinterpret_cast<const uint16_t*>(rp)[at]);
+                                }
+                            }
+                        } else {
+                            const int pitch = rows ? Geo::row_pitch(SF) : Geo::raw_w(SF) * fmt_bytes(SF);
+                            const uint32_t sh = rows ? row_shift_elems(zterm, gy, J.nx, x0, xa, SF) : 0u;
+                            window<K, SF, false, false>(rs + rrow * pitch, 4 * g + fmt_xalign(SF) - R,
+                                                               sh, win);
+                            if (!xin) clamp_window<K>(win, x0 + 4 * g, J.nx);
                         }
                         float4 o;
                         float* op = &o.x;
@@ -307,11 +329,21 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
                 failed = true;
                 return;
             }
-            if (tid == 0 && it + NS < nplanes) {
+            if (rows && tid == 0 && pend >= 0) {
+                mbar_arrive(&bars[pend]);
+                ++issued;
+            }
+            pend = -1;
+            if (tma && tid == 0 && it + NS < nplanes) {
                 mbar_arrive_expect_tx(&bars[s], txb);
                 tma_load_3d(raw + s * rawb, tmap, &bars[s], x0 - xa, y0 - R,
                             clampi(pfirst + it + NS, 0, J.nz - 1));
                 ++issued;
+            } else if (rows && it + NS < nplanes) {
+                // all threads; the arrival follows the next plane's barrier
+                copy_rows<Geo, BULK>(raw + s * rawb, &bars[s], J.src, vol_bytes, sfmt, J.nx, J.ny,
+                                    J.nz, x0, y0, pfirst + it + NS, tid);
+                pend = s;
             }
         } else {
         if (tma || rows) {
@@ -341,7 +373,7 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
             ++issued;
         } else if (rows && it + NS < nplanes) {
             // all threads; the arrival follows the x-pass barrier below
-            issue_rows<Geo, NT>(raw + s * rawb, &bars[s], J.src, vol_bytes, sfmt, J.nx, J.ny,
+            copy_rows<Geo, BULK>(raw + s * rawb, &bars[s], J.src, vol_bytes, sfmt, J.nx, J.ny,
                                 J.nz, x0, y0, pfirst + it + NS, tid);
         }
         // x pass: T1[row][x] = sum_a gx[a] F[row][x + a], 4 outputs per item
@@ -494,10 +526,16 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
     }
     // only bricks loaded through the stage barriers move them through their phases
     if (tma || rows) gplane = g0 + nplanes;
+    if (!tma) fence_proxy_async();   // a next brick's tensor-map loads may refill these stages
 
     if (failed) {
         if (tid == 0) {
             atomicOr(status, STATUS_TIMEOUT);
+            // a refill whose copies are in flight still needs its arrival before the drain
+            if (pend >= 0) {
+                mbar_arrive(&bars[pend]);
+                ++issued;
+            }
             for (int it = issued - 1; it >= 0 && it >= issued - NS; --it)
                 mbar_wait(&bars[(g0 + it) % NS], ((g0 + it) / NS) & 1);
         }
@@ -526,7 +564,7 @@ __host__ __device__ constexpr size_t smem_bytes_comp(int sfmt, bool rows = false
            static_cast<size_t>(Geo::FH) * tile_x<BXG>() * sizeof(float2);  // (hi, lo) x pass
 }
 
-template <int K, class Wt, int LM = LM_ANY, bool ROI = false, int BXG = BX>
+template <int K, class Wt, int LM = LM_ANY, bool ROI = false, int BXG = BX, bool BULK = false>
 __device__ __forceinline__ bool brick_comp(const Job& J, const Wt& G, const CUtensorMap* tmap,
                                            int bx, int by, int bz, unsigned char* smem,
                                            uint32_t& gplane, unsigned* status)
@@ -573,7 +611,7 @@ __device__ __forceinline__ bool brick_comp(const Job& J, const Wt& G, const CUte
     } else if (rows) {
         for (int s = 0; s < STAGES && s < nplanes; ++s) {
             const uint32_t q = g0 + s;
-            issue_rows<Geo, NT>(raw + (q % STAGES) * rawb, &bars[q % STAGES], J.src, vol_bytes,
+            copy_rows<Geo, BULK>(raw + (q % STAGES) * rawb, &bars[q % STAGES], J.src, vol_bytes,
                                 J.sfmt, J.nx, J.ny, J.nz, x0, y0, pfirst + s, tid);
         }
         __syncthreads();   // every thread's expect_tx precedes the single arrival
@@ -628,7 +666,7 @@ __device__ __forceinline__ bool brick_comp(const Job& J, const Wt& G, const CUte
             ++issued;
         } else if (rows && it + STAGES < nplanes) {
             // all threads; the arrival follows the x-pass barrier below
-            issue_rows<Geo, NT>(raw + s * rawb, &bars[s], J.src, vol_bytes, J.sfmt, J.nx, J.ny,
+            copy_rows<Geo, BULK>(raw + s * rawb, &bars[s], J.src, vol_bytes, J.sfmt, J.nx, J.ny,
                                 J.nz, x0, y0, pfirst + it + STAGES, tid);
         }
         // x pass (inputs exact): T1[row][x] = Dot2(gx, F[row][x .. x+k-1])
@@ -714,6 +752,7 @@ __device__ __forceinline__ bool brick_comp(const Job& J, const Wt& G, const CUte
 #pragma unroll 1
     for (int it = 0; it < nplanes && !failed; ++it) plane(it);
     if (tma || rows) gplane = g0 + nplanes;
+    if (!tma) fence_proxy_async();   // a next brick's tensor-map loads may refill these stages
     if (failed) {
         if (tid == 0) {
             atomicOr(status, STATUS_TIMEOUT);

@@ -27,6 +27,7 @@
 #pragma once
 
 #include "vkt_sep_brick.cuh"
+#include "vkt_split_plan.h"
 #include "vkt_window.cuh"
 
 namespace vkt {
@@ -45,15 +46,46 @@ struct SplitW {
     float a0h, a0l, a1h, a1l, qmax;
 };
 
-constexpr int SPLIT_LIST = 512;    // listed voxels that are worked off once there are as many
+// The split weights of the vectors g with the mapping of job J, where make_split_plan accepts them.
+template <int K>
+bool split_weights(const Job& J, const float* const g[3], SplitW<K>& S)
+{
+    SplitPlan p;
+    if (!make_split_plan(p, K, g, J.sfmt, J.a0, J.a0lo, J.a1, J.a1lo)) return false;
+    for (int i = 0; i < K; ++i) {
+        S.xh[i] = make_float2(p.hi[0][i], p.hi[0][i]);
+        S.xl[i] = make_float2(p.lo[0][i], p.lo[0][i]);
+        S.yh[i] = make_float2(p.hi[1][i], p.hi[1][i]);
+        S.yl[i] = make_float2(p.lo[1][i], p.lo[1][i]);
+        S.yw[i] = make_float2(g[1][i], g[1][i]);
+        S.zh[i] = make_float2(p.hi[2][i], p.hi[2][i]);
+        S.zl[i] = make_float2(p.lo[2][i], p.lo[2][i]);
+        S.zw[i] = make_float2(p.zg[i], p.zg[i]);
+        for (int a = 0; a < 3; ++a) S.g[a][i] = g[a][i];
+    }
+    S.my = p.my;
+    S.mz = p.mz;
+    S.whole = p.whole;
+    S.frac = p.frac;
+    S.tie = p.tie;
+    S.a0h = J.a0;
+    S.a0l = J.a0lo;
+    S.a1h = J.a1;
+    S.a1l = J.a1lo;
+    S.qmax = J.qmax;
+    return true;
+}
+
+constexpr int SPLIT_LIST = 512;    // listed voxels that are worked off once there are as many,
+constexpr int SPLIT_CHECK = 4;     // looked at every so many planes
 
 template <int K>
 __host__ __device__ constexpr size_t smem_bytes_split(int sfmt, bool rows = false)
 {
     using Geo = Brick<K, TX, CTY>;
     return 128 + static_cast<size_t>(STAGES) * Geo::stage_bytes(sfmt, rows) +
-           2 * static_cast<size_t>(Geo::FH) * TX * 2 * sizeof(float) +     // two (h, l) tiles
-           (SPLIT_LIST + TX * CTY) * sizeof(uint32_t) + 16;                // list, its length
+           3 * static_cast<size_t>(Geo::FH) * TX * 2 * sizeof(float) +     // three (h, l) tiles
+           (SPLIT_LIST + SPLIT_CHECK * TX * CTY) * sizeof(uint32_t) + 16;  // list, its length
 }
 
 // The code of voxel (x, y, z) by the operations of brick_comp, in its order.
@@ -162,10 +194,10 @@ __device__ __noinline__ unsigned dot2_voxel_warp(const void* src, int nx, int ny
     return comp_code(zs, zc, G.a0h, G.a0l, G.a1h, G.a1l, G.qmax);
 }
 
-template <int K, int SF, class Wt, int LM = LM_ANY, bool ROI = false, bool ROTZ = true>
+template <int K, int SF, class Wt, int LM = LM_ANY, bool ROI = false, bool ROTZ = true, bool BULK = false>
 __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUtensorMap* tmap,
                                             int bx, int by, int bz, unsigned char* smem,
-                                            uint32_t& gplane, unsigned* status)
+                                            uint32_t& gplane, uint32_t& xphase, unsigned* status)
 {
     __builtin_assume(threadIdx.x < NT);   // every launch of a brick has NT threads
     using Geo = Brick<K, TX, CTY>;
@@ -181,9 +213,11 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
     const int pitch = rows ? Geo::row_pitch(SF) : Geo::raw_w(SF) * ES;
     constexpr uint32_t txb = Geo::raw_tx(SF);
     unsigned char* raw = smem + 128;
-    float* T = reinterpret_cast<float*>(raw + STAGES * rawb);   // tile [plane & 1][h, l][FH][TX]
-    uint32_t* list = reinterpret_cast<uint32_t*>(T + 4 * FH * TX);
-    volatile uint32_t* count = list + SPLIT_LIST + TX * CTY;
+    float* T = reinterpret_cast<float*>(raw + STAGES * rawb);   // tile [plane % 3][h, l][FH][TX]
+    uint32_t* list = reinterpret_cast<uint32_t*>(T + 6 * FH * TX);
+    volatile uint32_t* count = list + SPLIT_LIST + SPLIT_CHECK * TX * CTY;
+    uint64_t* xbar = &bars[XBAR];
+    const uint32_t gx = xphase;
 
     const int tid = threadIdx.x;
     const int tx = tid % BX, ty = tid / BX;
@@ -195,7 +229,8 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
     const int nplanes = zc1 - zc0 + 2 * R;
     const uint32_t g0 = gplane;
 
-    if (tid == 0) *count = 0;   // read after the first plane's barrier
+    if (tid == 0) *count = 0;
+    __syncthreads();   // before a voxel is listed
     int issued = 0;
     const uint64_t vol_bytes = static_cast<uint64_t>(J.nx) * J.ny * J.nz * ES;
     if (tma && tid == 0) {
@@ -208,7 +243,7 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
     } else if (rows) {
         for (int s = 0; s < STAGES && s < nplanes; ++s) {
             const uint32_t q = g0 + s;
-            issue_rows<Geo, NT>(raw + (q % STAGES) * rawb, &bars[q % STAGES], J.src, vol_bytes, SF,
+            copy_rows<Geo, BULK>(raw + (q % STAGES) * rawb, &bars[q % STAGES], J.src, vol_bytes, SF,
                                 J.nx, J.ny, J.nz, x0, y0, pfirst + s, tid);
         }
         __syncthreads();   // every thread's expect_tx precedes the single arrival
@@ -253,7 +288,8 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
         }
     };
 
-    auto plane = [&](const int it, const int u) {
+    // The x pass of plane `it` into tile it % 3.
+    auto x_pass = [&](const int it) {
         const uint32_t q = g0 + it;
         const int s = q % STAGES;
         const unsigned char* rs = raw + s * rawb;
@@ -265,7 +301,7 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
                                     y0, pfirst + it, tid);
             __syncthreads();
         }
-        float* Th = T + (it & 1) * 2 * FH * TX;
+        float* Th = T + (it % 3) * 2 * FH * TX;
         float* Tl = Th + FH * TX;
         if (ok) {
             const uint32_t zterm = static_cast<uint32_t>(clampi(pfirst + it, 0, J.nz - 1)) *
@@ -301,18 +337,25 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
                 }
             }
         }
-        // the stage is read, the tile written, and every voxel of the planes before is listed:
-        // whoever lists the last of SPLIT_LIST voxels sees the full count here
-        if (__syncthreads_or(!ok || *count >= SPLIT_LIST)) {
-            if (__syncthreads_or(!ok)) {
-                failed = true;
-                return;
-            }
-            work_off();
-            __syncthreads();
-            if (tid == 0) *count = 0;
-            __syncthreads();
+        __syncwarp();
+        if ((tid & 31) == 0) mbar_arrive(xbar);
+        return ok;
+    };
+
+    // Plane `it`: the x pass of the plane after it, then its own y and z passes.  A warp arrives at
+    // xbar when its x pass of a plane is written and waits there one plane later, after the y and
+    // z passes in between, so the uneven x pass (FH * 16 items on 256 threads) and whatever else
+    // delays a warp is waited for only if it lasts longer than those.  With three tiles the wait
+    // for plane `it` also says that tile (it + 1) % 3 is free: a warp that has arrived for plane
+    // `it` is done with plane it - 2.
+    auto plane = [&](const int it, const int u) {
+        const uint32_t q = g0 + it;
+        const int s = q % STAGES;
+        if (!mbar_wait(xbar, (gx + it) & 1)) {
+            failed = true;
+            return;
         }
+        // stage s is read
         if (rows && tid == 0 && pend >= 0) {
             mbar_arrive(&bars[pend]);
             ++issued;
@@ -324,11 +367,23 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
                         clampi(pfirst + it + STAGES, 0, J.nz - 1));
             ++issued;
         } else if (rows && it + STAGES < nplanes) {
-            // all threads; the arrival follows the next plane's barrier
-            issue_rows<Geo, NT>(raw + s * rawb, &bars[s], J.src, vol_bytes, SF, J.nx, J.ny, J.nz, x0,
+            // all threads; the arrival follows the next plane's wait
+            copy_rows<Geo, BULK>(raw + s * rawb, &bars[s], J.src, vol_bytes, SF, J.nx, J.ny, J.nz, x0,
                                 y0, pfirst + it + STAGES, tid);
             pend = s;
         }
+        if (it % SPLIT_CHECK == SPLIT_CHECK - 1 && __syncthreads_or(*count >= SPLIT_LIST)) {
+            work_off();
+            __syncthreads();
+            if (tid == 0) *count = 0;
+            __syncthreads();
+        }
+        if (it + 1 < nplanes && !x_pass(it + 1)) {
+            failed = true;
+            return;
+        }
+        const float* Th = T + (it % 3) * 2 * FH * TX;
+        const float* Tl = Th + FH * TX;
         // y pass
         float2 H[RX / 2], L[RX / 2];
 #pragma unroll
@@ -403,6 +458,7 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
                 }
         }
     };
+    failed = !x_pass(0);
     if constexpr (ROTZ) {
 #pragma unroll 1
         for (int it = 0; it < nplanes && !failed; ++it) plane(it, 0);
@@ -417,7 +473,12 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
         }
     }
     if (tma || rows) gplane = g0 + nplanes;
+    xphase = gx + nplanes;
+    if (!tma) fence_proxy_async();   // a next brick's tensor-map loads may refill these stages
+    // (all threads wait for the same stages and for one another, so they fail together, within the
+    // limit of a wait)
     if (failed) {
+        __syncthreads();
         if (tid == 0) {
             atomicOr(status, STATUS_TIMEOUT);
             // a refill whose copies are in flight still needs its arrival before the drain

@@ -9,16 +9,15 @@
 
 #include "vkt_sep_brick.cuh"
 #include "vkt_sep_split.cuh"
-#include "vkt_split_plan.h"
 
 namespace vkt {
 namespace sepk {
 
 // CTAs per SM the register allocation must allow: three up to k = 5 (the float32 and
-// run-time-format kernels fit in 80 registers there), two for k = 7 and for the uint8
+// run-time-format kernels fit in 80 registers there), two for k = 7 and for the integer
 // kernels, whose fused word-load x pass needs about 120
 template <int K, int SF>
-constexpr int sep_min_blocks() { return (K <= 5 && SF != FMT_U8) ? 3 : 2; }
+constexpr int sep_min_blocks() { return (K <= 5 && SF != FMT_U8 && SF != FMT_U16) ? 3 : 2; }
 
 // planes in flight of a single-volume kernel: k for whole-volume tensor-map kernels up to
 // k = 7, a ring whose stage and phase are compile-time constants of the k-times unrolled
@@ -78,44 +77,9 @@ __global__ void __launch_bounds__(sep::NT, 2)   // three per SM: 365 against 337
     __syncthreads();
     grid_dependency_wait();   // programmatic launch: the previous kernel's writes are visible
     launch_dependents();
-    uint32_t gplane = 0;
+    uint32_t gplane = 0, xphase = 0;
     sep::brick_split<K, SF, sep::SplitW<K>, LM, ROI, (K > 5 || LM != sep::LM_TMA)>(J, G, &tmap, blockIdx.x, blockIdx.y, blockIdx.z,
-                                                     smem, gplane, status);
-}
-
-// The split weights of a job, where the split evaluation suits it: k >= 3 (at k = 1 Dot2 is
-// three products), integer sources (a float32 voxel has no unit that the weights' parts could
-// be exact in), and a filter that make_split_plan accepts.  512 x 512 x 256 uint16, k = 5:
-// 635 us by Dot2, 311 us by the split.
-template <int K>
-bool split_weights(const sep::Job& J, const sep::W<K>& G, sep::SplitW<K>& S)
-{
-    if (K < 3 || !J.comp || J.sfmt == FMT_F32) return false;
-    SplitPlan p;
-    const float* const g[3] = {G.gx, G.gy, G.gz};
-    if (!make_split_plan(p, K, g, J.sfmt, J.a0, J.a0lo, J.a1, J.a1lo)) return false;
-    for (int i = 0; i < K; ++i) {
-        S.xh[i] = make_float2(p.hi[0][i], p.hi[0][i]);
-        S.xl[i] = make_float2(p.lo[0][i], p.lo[0][i]);
-        S.yh[i] = make_float2(p.hi[1][i], p.hi[1][i]);
-        S.yl[i] = make_float2(p.lo[1][i], p.lo[1][i]);
-        S.yw[i] = make_float2(g[1][i], g[1][i]);
-        S.zh[i] = make_float2(p.hi[2][i], p.hi[2][i]);
-        S.zl[i] = make_float2(p.lo[2][i], p.lo[2][i]);
-        S.zw[i] = make_float2(p.zg[i], p.zg[i]);
-        for (int a = 0; a < 3; ++a) S.g[a][i] = g[a][i];
-    }
-    S.my = p.my;
-    S.mz = p.mz;
-    S.whole = p.whole;
-    S.frac = p.frac;
-    S.tie = p.tie;
-    S.a0h = J.a0;
-    S.a0l = J.a0lo;
-    S.a1h = J.a1;
-    S.a1l = J.a1lo;
-    S.qmax = J.qmax;
-    return true;
+                                                     smem, gplane, xphase, status);
 }
 
 // the kernel for a job: tensor-map jobs and (for the compiled-in formats) row-copy jobs get
@@ -182,16 +146,28 @@ vktError launch_k(const Job& job, const float* gx, const float* gy, const float*
                                      Geo::raw_w(job.sfmt), ty + 2 * Geo::R, 1)
                     ? 1
                     : 0;
-    // rows that no tensor map can describe are still fetched asynchronously, one bulk copy
-    // per row, when the volume starts on a 16-byte boundary
+    // rows that no tensor map can describe are still fetched asynchronously, as 16-byte
+    // blocks, when the volume starts on a 16-byte boundary
     J.rows = (!J.use_tma && reinterpret_cast<uintptr_t>(J.src) % 16 == 0) ? 1 : 0;
     if (!J.use_tma) memset(&map, 0, sizeof(map));
     size_t smem = J.comp ? sep::smem_bytes_comp<K>(job.sfmt, J.rows != 0)
                          : sep::smem_bytes<K>(job.sfmt, J.rows != 0);
     // the common float32 destinations get kernels with their formats compiled in
     auto fast = pick_fast<K, -1, -1>(J);
+    bool fx = false;   // the fused x pass (its own shared-memory layout)
     if constexpr (K >= 3 && K <= 7) {
-        if (!J.comp && J.dfmt == FMT_F32 && J.sfmt == FMT_U8) fast = pick_fast<K, FMT_U8, FMT_F32>(J);
+        // integer sources read their windows as words however they are loaded
+        if (!J.comp && J.sfmt == FMT_U8)
+            fast = J.use_tma ? (J.dfmt == FMT_F32 ? k_separable<K, FMT_U8, FMT_F32, sep::LM_TMA>
+                                                  : k_separable<K, FMT_U8, -1, sep::LM_TMA>)
+                   : J.rows  ? (J.dfmt == FMT_F32 ? k_separable<K, FMT_U8, FMT_F32, sep::LM_ROWS>
+                                                  : k_separable<K, FMT_U8, -1, sep::LM_ROWS>)
+                             : k_separable<K, FMT_U8, -1, sep::LM_ANY>;
+        if (!J.comp && J.sfmt == FMT_U16)
+            fast = J.use_tma ? k_separable<K, FMT_U16, -1, sep::LM_TMA>
+                   : J.rows  ? k_separable<K, FMT_U16, -1, sep::LM_ROWS>
+                             : k_separable<K, FMT_U16, -1, sep::LM_ANY>;
+        fx = !J.comp && (J.sfmt == FMT_F32 ? J.use_tma && J.dfmt == FMT_F32 : J.use_tma || K <= 5);
         if (!J.comp && J.dfmt == FMT_F32 && J.sfmt == FMT_F32) fast = pick_fast<K, FMT_F32, FMT_F32>(J);
     }
     auto comp = J.use_tma ? k_separable_comp<K, sep::LM_TMA> : k_separable_comp<K, sep::LM_ANY>;
@@ -201,26 +177,27 @@ vktError launch_k(const Job& job, const float* gx, const float* gy, const float*
         fast = k_separable<K, -1, -1, sep::LM_ANY, true>;
         comp = k_separable_comp<K, sep::LM_ANY, true>;
         if constexpr (K >= 3 && K <= 7) {
+            if (!J.comp && J.sfmt == FMT_U8) fast = k_separable<K, FMT_U8, -1, sep::LM_ANY, true>;
+            if (!J.comp && J.sfmt == FMT_U16) fast = k_separable<K, FMT_U16, -1, sep::LM_ANY, true>;
             if (!J.comp && J.use_tma && J.dfmt == FMT_F32 && J.sfmt == FMT_U8)
                 fast = k_separable<K, FMT_U8, FMT_F32, sep::LM_TMA, true>;
             if (!J.comp && J.use_tma && J.dfmt == FMT_F32 && J.sfmt == FMT_F32)
                 fast = k_separable<K, FMT_F32, FMT_F32, sep::LM_TMA, true>;
         }
     }
-    // the tensor-map kernels of the compiled-in formats fuse the conversion into the x pass
-    // (their own shared-memory layout)
-    if (!J.comp && J.use_tma && J.dfmt == FMT_F32 &&
-        (J.sfmt == FMT_F32 || J.sfmt == FMT_U8) && K >= 3 && K <= 7)
-        smem = std::max(smem, sep::smem_bytes_fx<K, K>(job.sfmt));
+    if (fx) smem = std::max(smem, sep::smem_bytes_fx<K, K>(job.sfmt, J.rows != 0));
     if (!J.comp && J.use_tma && !job.roi && K >= 3 && K <= 7)
         smem = std::max(smem, sep::smem_bytes<K, K>(job.sfmt, false));
-    // integer sources whose codes need more than FP32: the split evaluation where it suits the
-    // filter, else Dot2
+    // Integer codes that need more than FP32: the split evaluation where it suits the job, else
+    // Dot2.  k >= 3 (at k = 1 Dot2 is three products), integer sources (a float32 voxel has no unit
+    // that the weights' parts could be exact in), and a filter that make_split_plan accepts.
+    // 512 x 512 x 256 uint16, k = 5: 635 us by Dot2, 311 us by the split.
     sep::SplitW<K> S;
     bool use_split = false;
     auto split = &k_separable_split<(K < 3 ? 3 : K), FMT_U16, sep::LM_ANY, true>;
     if constexpr (K >= 3) {
-        use_split = split_weights<K>(J, G, S);
+        const float* const g[3] = {G.gx, G.gy, G.gz};
+        use_split = J.comp && J.sfmt != FMT_F32 && sep::split_weights<K>(J, g, S);
         if (J.sfmt == FMT_U8) split = k_separable_split<K, FMT_U8, sep::LM_ANY, true>;
         else if (!job.roi) split = J.use_tma ? k_separable_split<K, FMT_U16, sep::LM_TMA>
                                              : k_separable_split<K, FMT_U16, sep::LM_ANY>;

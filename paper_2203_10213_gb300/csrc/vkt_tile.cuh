@@ -193,25 +193,70 @@ struct Brick {
 
 // Row-copy loading, for volumes whose rows are not a multiple of 16 bytes long (no tensor
 // map can describe them).  Stage row r (r < FH, global row y0 - R + r inside the volume) is
-// filled by one 1-D bulk copy of the 16-byte aligned span around raw columns
+// filled by 16-byte asynchronous copies of the 16-byte blocks that cover raw columns
 // [0, raw_w) = voxels [x0 - xa, x0 - xa + raw_w) of plane clamp(z); the raw column 0 of the
 // row lands at the row's misalignment (row_shift_elems) in the stage row.  Rows outside the
-// volume are not copied: the clamped conversion never reads them.  The copies are clipped
-// to the volume's full 16-byte blocks, so no byte outside the volume is read; the few bytes
-// of the last partial block a row needs are read with plain loads.
+// volume are not copied: the clamped conversion never reads them.  Only the volume's full
+// 16-byte blocks are copied, so no byte outside the volume is read; the few bytes of the
+// last partial block a row needs are read with plain loads.
 //
-// Every thread of the CTA calls issue_rows; thread (lane l, warp w) takes row 8 l + w, so
-// the rows spread over the warps.  Each copying thread first adds its bytes to the stage
-// barrier's transaction count (expect_tx, no arrival), then starts its copy.  The caller
-// makes the barrier's single arrival (rows_arrive) from one thread after a CTA barrier that
-// follows every thread's issue_rows, so the phase cannot complete before all bytes are
-// expected, and the plain-loaded bytes are visible to whoever waits on the phase.
+// Every thread of the CTA calls issue_rows and copies about one block per plane (a uint8 plane
+// of 36 rows has 252).  Its copies' completion is added to the stage barrier's pending count
+// before the call returns (cp.async.mbarrier.arrive).  The caller makes the barrier's single
+// arrival (rows_arrive) from one thread after a CTA barrier that follows every thread's
+// issue_rows, so the phase cannot complete before all copies are counted, and the
+// plain-loaded bytes are visible to whoever waits on the phase.
+// (One bulk copy per row, issue_rows_bulk, makes the kernels wait for the copy unit, which takes
+// these 112-byte copies one at a time: 302^3 uint8, k = 5, into uint8 97 us against 88, into float32
+// 87 against 78.  The batch, with several kernels' bricks on an SM, has work for that time and
+// spends fewer instructions with it: 570 against 584 us for 128 mixed volumes.)
 __device__ __forceinline__ uint32_t row_shift_elems(uint32_t zterm, int gy, int nx, int x0, int xa,
                                                     int fmt)
 {
     const uint32_t mask = static_cast<uint32_t>(16 / fmt_bytes(fmt)) - 1u;
     return (zterm + static_cast<uint32_t>(gy) * static_cast<uint32_t>(nx) +
             static_cast<uint32_t>(x0 - xa)) & mask;
+}
+
+__device__ __forceinline__ void copy_async_16(void* dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)),
+                 "l"(reinterpret_cast<uint64_t>(src))
+                 : "memory");
+}
+
+// the thread's asynchronous copies so far become one more pending arrival of the barrier's
+// current phase, made when they are complete
+__device__ __forceinline__ void mbar_arrive_on_copies(uint64_t* bar)
+{
+    asm volatile("cp.async.mbarrier.arrive.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+template <typename Geo, int NT>
+__device__ __forceinline__ void issue_rows(unsigned char* stage, uint64_t* bar, const void* src,
+                                           uint64_t vol_bytes, int fmt, int nx, int ny, int nz,
+                                           int x0, int y0, int z, int tid)
+{
+    const int es = fmt_bytes(fmt);
+    const int xa = fmt_xalign(fmt);
+    const int need = Geo::raw_w(fmt) * es;      // a multiple of 16
+    const int blocks = need / 16 + 1;           // of a row at any misalignment
+    const unsigned char* base = static_cast<const unsigned char*>(src);
+    const int64_t plane = static_cast<int64_t>(clampi(z, 0, nz - 1)) * ny;
+    for (int i = tid; i < Geo::FH * blocks; i += NT) {
+        const int r = i / blocks, c = i - r * blocks;
+        const int yy = y0 - Geo::R + r;
+        if (yy < 0 || yy >= ny) continue;
+        const int64_t b0 = ((plane + yy) * nx + (x0 - xa)) * es;
+        const int64_t at = (b0 & ~int64_t(15)) + 16 * c;    // floored to 16 bytes (also below 0)
+        if (at < 0 || at >= b0 + need) continue;
+        unsigned char* to = stage + r * Geo::row_pitch(fmt) + 16 * c;
+        if (at + 16 <= static_cast<int64_t>(vol_bytes))
+            copy_async_16(to, base + at);
+        else
+            for (int64_t e = at; e < static_cast<int64_t>(vol_bytes); ++e) to[e - at] = __ldg(base + e);
+    }
+    mbar_arrive_on_copies(bar);
 }
 
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes)
@@ -221,8 +266,10 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes)
                  : "memory");
 }
 
+// The same by one bulk copy per row, thread (lane l, warp w) taking row 8 l + w: a bulk copy's
+// bytes are added to the barrier's transaction count before it starts.
 template <typename Geo, int NT>
-__device__ __forceinline__ void issue_rows(unsigned char* stage, uint64_t* bar, const void* src,
+__device__ __forceinline__ void issue_rows_bulk(unsigned char* stage, uint64_t* bar, const void* src,
                                            uint64_t vol_bytes, int fmt, int nx, int ny, int nz,
                                            int x0, int y0, int z, int tid)
 {
@@ -425,6 +472,40 @@ __device__ __forceinline__ void load_row(const float* p, float (&v)[N])
     for (int i = N2; i < N; ++i) v[i] = p[i];
 }
 
+// Writes codes first .. nvalid-1 of RX consecutive ones from idx, whole groups of four as one
+// store where they are aligned.
+template <int RX>
+__device__ __forceinline__ void store_codes(void* dst, int dfmt, int64_t idx, int first, int nvalid,
+                                            const unsigned (&q)[RX])
+{
+    if (RX == 4 && first == 0 && nvalid >= 4) {
+        if (dfmt == FMT_U16) {
+            uint16_t* d = static_cast<uint16_t*>(dst) + idx;
+            if ((reinterpret_cast<uintptr_t>(d) & 7) == 0) {
+                *reinterpret_cast<uint2*>(d) = make_uint2(q[0] | (q[1] << 16), q[2] | (q[3] << 16));
+                return;
+            }
+        } else {
+            unsigned char* d = static_cast<unsigned char*>(dst) + idx;
+            if ((reinterpret_cast<uintptr_t>(d) & 3) == 0) {
+                *reinterpret_cast<uint32_t*>(d) = q[0] | (q[1] << 8) | (q[2] << 16) | (q[3] << 24);
+                return;
+            }
+        }
+    }
+    if (dfmt == FMT_U16) {
+        uint16_t* d = static_cast<uint16_t*>(dst) + idx;
+#pragma unroll
+        for (int x = 0; x < RX; ++x)
+            if (x >= first && x < nvalid) d[x] = static_cast<uint16_t>(q[x]);
+    } else {
+        unsigned char* d = static_cast<unsigned char*>(dst) + idx;
+#pragma unroll
+        for (int x = 0; x < RX; ++x)
+            if (x >= first && x < nvalid) d[x] = static_cast<unsigned char>(q[x]);
+    }
+}
+
 // Writes results first .. nvalid-1 of RX consecutive results of one row (from idx), mapped
 // to the destination format.
 template <int RX>
@@ -451,17 +532,7 @@ __device__ __forceinline__ void store_row(void* dst, int dfmt, int64_t idx, int 
     unsigned q[RX];
 #pragma unroll
     for (int x = 0; x < RX; ++x) q[x] = static_cast<unsigned>(fminf(fmaxf(rintf(v[x]), 0.f), qmax));
-    if (dfmt == FMT_U16) {
-        uint16_t* d = reinterpret_cast<uint16_t*>(dst) + idx;
-#pragma unroll
-        for (int x = 0; x < RX; ++x)
-            if (x >= first && x < nvalid) d[x] = static_cast<uint16_t>(q[x]);
-    } else {
-        unsigned char* d = reinterpret_cast<unsigned char*>(dst) + idx;
-#pragma unroll
-        for (int x = 0; x < RX; ++x)
-            if (x >= first && x < nvalid) d[x] = static_cast<unsigned char>(q[x]);
-    }
+    store_codes<RX>(dst, dfmt, idx, first, nvalid, q);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -1,6 +1,6 @@
 // vkt_window.cuh -- the x pass's window of an integer source, read from a raw stage as aligned
 // 32-bit words, for every way a stage is filled (one TMA box, row copies at any misalignment,
-// plain loads), and the store of a row of codes.
+// plain loads).
 //
 // A window of K + 3 codes (four outputs) is 8 to 24 bytes: two to seven word loads and at most
 // one funnel shift per word, instead of K + 3 one-element loads.  The clamp at the volume's x
@@ -73,40 +73,6 @@ __device__ __forceinline__ void clamp_window(float (&win)[K + 3], int gx, int nx
     const int last = nx - 1 - gx + R;      // the window index of voxel nx - 1
 #pragma unroll
     for (int e = 1; e < K + 3; ++e) win[e] = e > last ? win[e - 1] : win[e];
-}
-
-// Writes codes first .. nvalid-1 of RX consecutive ones from idx, whole groups of four as one
-// store where they are aligned.
-template <int RX>
-__device__ __forceinline__ void store_codes(void* dst, int dfmt, int64_t idx, int first, int nvalid,
-                                            const unsigned (&q)[RX])
-{
-    if (RX == 4 && first == 0 && nvalid >= 4) {
-        if (dfmt == FMT_U16) {
-            uint16_t* d = static_cast<uint16_t*>(dst) + idx;
-            if ((reinterpret_cast<uintptr_t>(d) & 7) == 0) {
-                *reinterpret_cast<uint2*>(d) = make_uint2(q[0] | (q[1] << 16), q[2] | (q[3] << 16));
-                return;
-            }
-        } else {
-            unsigned char* d = static_cast<unsigned char*>(dst) + idx;
-            if ((reinterpret_cast<uintptr_t>(d) & 3) == 0) {
-                *reinterpret_cast<uint32_t*>(d) = q[0] | (q[1] << 8) | (q[2] << 16) | (q[3] << 24);
-                return;
-            }
-        }
-    }
-    if (dfmt == FMT_U16) {
-        uint16_t* d = static_cast<uint16_t*>(dst) + idx;
-#pragma unroll
-        for (int x = 0; x < RX; ++x)
-            if (x >= first && x < nvalid) d[x] = static_cast<uint16_t>(q[x]);
-    } else {
-        unsigned char* d = static_cast<unsigned char*>(dst) + idx;
-#pragma unroll
-        for (int x = 0; x < RX; ++x)
-            if (x >= first && x < nvalid) d[x] = static_cast<unsigned char>(q[x]);
-    }
 }
 
 }  // namespace vkt
