@@ -19,9 +19,11 @@
 #include <cstring>
 #include <list>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "vkt_sep_brick.cuh"
+#include "vkt_sep_split.cuh"
 
 namespace vkt {
 namespace {
@@ -33,12 +35,13 @@ namespace {
 // parallel branches of the graph: blocks of the next kernel fill the SMs that a drained
 // kernel leaves, so no kernel's tail idles the GPU.
 using BatchKernel = void (*)(const sep::Job*, const CUtensorMap*, const int4*, int, unsigned*,
-                             unsigned*);
+                             unsigned*, const unsigned char*);
 
 template <int K, bool COMP, int BXG>
 __global__ void __launch_bounds__(sep::NT, 2)
     k_sep_batch(const sep::Job* __restrict__ jobs, const CUtensorMap* __restrict__ maps,
-                const int4* __restrict__ items, int nitems, unsigned* counter, unsigned* status)
+                const int4* __restrict__ items, int nitems, unsigned* counter, unsigned* status,
+                const unsigned char*)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int next;
@@ -63,12 +66,50 @@ __global__ void __launch_bounds__(sep::NT, 2)
         }
         bool ok;
         if constexpr (COMP)
-            ok = sep::brick_comp<K, sep::W<K>, sep::LM_ANY, false, BXG>(J, G, tm, w.y, w.z, w.w, smem,
+            ok = sep::brick_comp<K, sep::W<K>, sep::LM_ANY, false, BXG, true>(J, G, tm, w.y, w.z, w.w, smem,
                                                                         gplane, status);
         else
             ok = sep::brick<K, sep::W<K>, -1, -1, sep::LM_ANY, false, sep::FSTAGES, false, (K >= 5),
-                            BXG>(J, G, tm, w.y, w.z, w.w, smem, gplane, status);
+                            BXG, true>(J, G, tm, w.y, w.z, w.w, smem, gplane, status);
         if (!ok) break;
+    }
+}
+
+// The split evaluation (vkt_sep_split.cuh) of uint16 volumes: each volume's split weights stand in
+// a table of its own and are staged in shared memory for its bricks (as registers they and the
+// accumulators would not fit, and one launch's constants cannot hold every volume's).
+constexpr size_t SPLIT_PITCH = sizeof(sep::SplitW<7>);   // bytes from one volume's to the next
+
+template <int K>
+__global__ void __launch_bounds__(sep::NT, 2)
+    k_sep_batch_split(const sep::Job* __restrict__ jobs, const CUtensorMap* __restrict__ maps,
+                      const int4* __restrict__ items, int nitems, unsigned* counter, unsigned* status,
+                      const unsigned char* weights)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ int next;
+    __shared__ sep::SplitW<K> G;
+    if (threadIdx.x == 0) sep::init_barriers(smem);
+    __syncthreads();
+    uint32_t gplane = 0, xphase = 0;
+    int held = -1;   // the volume whose weights G holds
+    for (;;) {
+        if (threadIdx.x == 0) next = static_cast<int>(atomicAdd(counter, 1u));
+        __syncthreads();
+        const int item = next;
+        __syncthreads();
+        if (item >= nitems) break;
+        const int4 w = items[item];
+        if (w.x != held) {
+            const uint32_t* from = reinterpret_cast<const uint32_t*>(weights + w.x * SPLIT_PITCH);
+            for (int i = threadIdx.x; i < static_cast<int>(sizeof(G) / 4); i += sep::NT)
+                reinterpret_cast<uint32_t*>(&G)[i] = from[i];
+            held = w.x;
+            __syncthreads();
+        }
+        if (!sep::brick_split<K, FMT_U16, sep::SplitW<K>, sep::LM_ANY, false, true, true>(jobs[w.x], G, maps + w.x, w.y, w.z, w.w, smem,
+                                                          gplane, xphase, status))
+            break;
     }
 }
 
@@ -91,8 +132,14 @@ BatchKernel kernel_of(int k, bool comp)
     }
 }
 
-BatchKernel batch_kernel(int k, bool comp, bool narrow)
+// How a volume is accumulated: FP32, Dot2, or split (uint16 into integer codes, default shape).
+enum : int { B_PLAIN = 0, B_DOT2 = 1, B_SPLIT = 2 };
+
+BatchKernel batch_kernel(int k, int mode, bool narrow)
 {
+    if (mode == B_SPLIT)
+        return k <= 3 ? k_sep_batch_split<3> : k <= 5 ? k_sep_batch_split<5> : k_sep_batch_split<7>;
+    const bool comp = mode == B_DOT2;
     return narrow ? kernel_of<BXN>(k, comp) : kernel_of<sep::BX>(k, comp);
 }
 
@@ -115,8 +162,12 @@ size_t smem_of(int k, int sfmt, bool comp, bool rows)
     }
 }
 
-size_t batch_smem(int k, int sfmt, bool comp, bool rows, bool narrow)
+size_t batch_smem(int k, int sfmt, int mode, bool rows, bool narrow)
 {
+    if (mode == B_SPLIT)
+        return k <= 3 ? sep::smem_bytes_split<3>(sfmt, rows)
+                      : k <= 5 ? sep::smem_bytes_split<5>(sfmt, rows) : sep::smem_bytes_split<7>(sfmt, rows);
+    const bool comp = mode == B_DOT2;
     return narrow ? smem_of<BXN>(k, sfmt, comp, rows) : smem_of<sep::BX>(k, sfmt, comp, rows);
 }
 
@@ -141,6 +192,41 @@ bool narrow_for(int nx, int ny, bool comp)
 // TMA box width (raw voxels per stage row) of a brick with tx outputs along x
 int raw_width(int tx, int sfmt) { return tx + 2 * fmt_xalign(sfmt); }
 
+// One volume's mode, and its split weights (SPLIT_PITCH bytes) where they are used.  Volumes of a
+// batch mostly share a few filters, so the last few answers are kept for the call (`seen`).
+struct Split {
+    float g[3][VKT_MAX_FILTER_SIZE];
+    float map[5];
+    int k;
+    bool ok;
+    std::vector<unsigned char> w;
+};
+
+const Split& split_of(std::list<Split>& seen, const sep::Job& J, int k)
+{
+    const float map[5] = {J.a0, J.a0lo, J.a1, J.a1lo, J.qmax};
+    for (const Split& s : seen)
+        if (s.k == k && memcmp(s.map, map, sizeof(map)) == 0 && memcmp(s.g, J.g, sizeof(s.g)) == 0) return s;
+    seen.emplace_front();
+    Split& s = seen.front();
+    memcpy(s.g, J.g, sizeof(s.g));
+    memcpy(s.map, map, sizeof(map));
+    s.k = k;
+    s.w.assign(SPLIT_PITCH, 0);
+    const float* const g[3] = {J.g[0], J.g[1], J.g[2]};
+    auto fill = [&](auto kc) {
+        sep::SplitW<decltype(kc)::value> W;
+        memset(&W, 0, sizeof(W));
+        s.ok = sep::split_weights<decltype(kc)::value>(J, g, W);
+        memcpy(s.w.data(), &W, sizeof(W));
+    };
+    s.ok = false;
+    if (k == 3) fill(std::integral_constant<int, 3>{});
+    if (k == 5) fill(std::integral_constant<int, 5>{});
+    if (k == 7) fill(std::integral_constant<int, 7>{});
+    return s;
+}
+
 // A replayable batch: device table, tensor maps, work list, counter, and the graph.
 struct Plan {
     std::vector<unsigned char> key;
@@ -150,7 +236,9 @@ struct Plan {
     CUtensorMap* d_maps = nullptr;
     int4* d_items = nullptr;
     unsigned* d_counter = nullptr;    // one work-list counter per persistent kernel
+    unsigned char* d_split = nullptr; // split weights, SPLIT_PITCH bytes per separable volume
     std::vector<sep::Job> jobs;       // table as last uploaded
+    std::vector<unsigned char> split; // split weights as last uploaded
     int nitems = 0;
     unsigned kernels = 0;             // kernels one replay launches
     cudaGraph_t graph = nullptr;
@@ -254,17 +342,16 @@ int batch_zchunk(int nz, int target)
 
 // sep_idx: triples for the persistent kernel; dense_idx: triples launched on their own
 // (dense filters, and separable ones of k = 9) inside the same graph.
-// zt: brick z extent target (batch_zchunk); per_sm_cap: CTAs per SM of the persistent grids
+// modes: B_* of each separable triple.  zt: brick z extent target (batch_zchunk); per_sm_cap: CTAs per SM of the persistent grids
 // (0: as many as the occupancy allows); narrow: volumes that the narrow brick covers with
 // less padding take it
 vktError build_plan(Plan& P, int32_t n, vktStructuredVolume* dst, vktStructuredVolume* src,
                     vktFilter* filters, const std::vector<int>& sep_idx,
-                    const std::vector<int>& dense_idx, bool force_dense, bool force_direct,
-                    const Ctx& ctx, int zt = 64, int per_sm_cap = 0, bool narrow = false)
+                    const std::vector<int>& dense_idx, const std::vector<int>& modes,
+                    const std::vector<const Split*>& splits, bool force_dense, bool force_direct, const Ctx& ctx, int zt = 64, int per_sm_cap = 0, bool narrow = false)
 {
     // work list: separable volumes' bricks, heavy kernels first
     std::vector<int4> items;
-    size_t smem = 0;
     P.jobs.resize(sep_idx.size());
     std::vector<CUtensorMap> maps(sep_idx.size());
     std::vector<char> vnarrow(sep_idx.size(), 0);   // the brick shape of each volume
@@ -283,8 +370,8 @@ vktError build_plan(Plan& P, int32_t n, vktStructuredVolume* dst, vktStructuredV
         J.sfmt = s->format;
         J.dfmt = dst[i]->format;
         J.k = filters[i]->k;
-        J.comp = separable_needs_comp(dst[i], s, filters[i]) ? 1 : 0;
-        vnarrow[j] = narrow && narrow_for(J.nx, J.ny, J.comp != 0);
+        J.comp = modes[j] != B_PLAIN ? 1 : 0;   // (the split brick has the compensated one's tile)
+        vnarrow[j] = narrow && modes[j] != B_SPLIT && narrow_for(J.nx, J.ny, J.comp != 0);
         const int tx = tile_x(vnarrow[j]), ty = tile_y(vnarrow[j], J.comp != 0);
         J.zchunk = batch_zchunk(J.nz, zt);
         J.tiles_x = (J.nx + tx - 1) / tx;
@@ -295,25 +382,25 @@ vktError build_plan(Plan& P, int32_t n, vktStructuredVolume* dst, vktStructuredV
                                          raw_width(tx, J.sfmt), ty + 2 * ((J.k - 1) / 2), 1)
                         ? 1
                         : 0;
-        // rows that no tensor map can describe are still fetched asynchronously, one bulk copy
-        // per row, when the volume starts on a 16-byte boundary
+        // rows that no tensor map can describe are still fetched asynchronously, as 16-byte
+        // blocks, when the volume starts on a 16-byte boundary
         J.rows = (!J.use_tma && reinterpret_cast<uintptr_t>(J.src) % 16 == 0) ? 1 : 0;
-        smem = std::max(smem, batch_smem(J.k, J.sfmt, J.comp != 0, J.rows != 0, vnarrow[j]));
         order.push_back({-static_cast<long>(J.k) * (J.zchunk + J.k - 1), static_cast<int>(j)});
     }
     std::stable_sort(order.begin(), order.end());
     // one work list per (K, mode), each ordered heavy bricks first
-    // list l = (k slot, mode, shape): (2 * k_slot + comp) * 2 + narrow
-    constexpr int NL = 4 * NKS;
+    // list l = (k slot, mode, shape): (3 * k_slot + mode) * 2 + narrow
+    constexpr int NL = 6 * NKS;
     std::vector<int4> lists[NL];
     size_t lsmem[NL] = {};
     double lwork[NL] = {};
     for (const auto& o : order) {
         const sep::Job& J = P.jobs[o.second];
-        const int l = (2 * k_slot(J.k) + (J.comp ? 1 : 0)) * 2 + (vnarrow[o.second] ? 1 : 0);
-        lsmem[l] = std::max(lsmem[l], batch_smem(J.k, J.sfmt, J.comp != 0, J.rows != 0,
-                                                 vnarrow[o.second]));
-        lwork[l] += static_cast<double>(J.nx) * J.ny * J.nz * J.k * (J.comp ? 10.0 : 1.0);
+        const int mode = modes[o.second];
+        const int l = (3 * k_slot(J.k) + mode) * 2 + (vnarrow[o.second] ? 1 : 0);
+        lsmem[l] = std::max(lsmem[l], batch_smem(J.k, J.sfmt, mode, J.rows != 0, vnarrow[o.second]));
+        lwork[l] += static_cast<double>(J.nx) * J.ny * J.nz * J.k *
+                    (mode == B_DOT2 ? 10.0 : mode == B_SPLIT ? 4.0 : 1.0);
         for (int bz = 0; bz < J.chunks; ++bz)
             for (int by = 0; by < J.tiles_y; ++by)
                 for (int bx = 0; bx < J.tiles_x; ++bx)
@@ -325,14 +412,14 @@ vktError build_plan(Plan& P, int32_t n, vktStructuredVolume* dst, vktStructuredV
         items.insert(items.end(), lists[l].begin(), lists[l].end());
     }
     P.nitems = static_cast<int>(items.size());
-    (void)smem;
 
     // one device block: table | maps (64-byte aligned) | items | one counter per list
     const size_t njobs = std::max<size_t>(1, P.jobs.size());
     const size_t off_maps = ((njobs * sizeof(sep::Job)) + 127) & ~size_t(127);
     const size_t off_items = off_maps + njobs * sizeof(CUtensorMap);
     const size_t off_counter = off_items + std::max<size_t>(1, items.size()) * sizeof(int4);
-    const size_t total = off_counter + 4 * NKS * 128;   // counters 128 bytes apart
+    const size_t off_split = off_counter + NL * 128;   // counters 128 bytes apart
+    const size_t total = off_split + njobs * SPLIT_PITCH;
     cudaError_t e = cudaMalloc(&P.dmem, total);
     if (e != cudaSuccess) return from_cuda(e);
     unsigned char* base = static_cast<unsigned char*>(P.dmem);
@@ -340,12 +427,18 @@ vktError build_plan(Plan& P, int32_t n, vktStructuredVolume* dst, vktStructuredV
     P.d_maps = reinterpret_cast<CUtensorMap*>(base + off_maps);
     P.d_items = reinterpret_cast<int4*>(base + off_items);
     P.d_counter = reinterpret_cast<unsigned*>(base + off_counter);
+    P.d_split = base + off_split;
+    // (the split weights go up at once: timed with zero weights every voxel would be listed)
+    P.split.assign(njobs * SPLIT_PITCH, 0);
+    for (size_t j = 0; j < P.jobs.size(); ++j)
+        if (modes[j] == B_SPLIT) memcpy(P.split.data() + j * SPLIT_PITCH, splits[j]->w.data(), SPLIT_PITCH);
     if (!P.jobs.empty()) {
         e = cudaMemcpy(P.d_jobs, P.jobs.data(), P.jobs.size() * sizeof(sep::Job), cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
             e = cudaMemcpy(P.d_maps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice);
         if (e == cudaSuccess && !items.empty())
             e = cudaMemcpy(P.d_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(P.d_split, P.split.data(), P.split.size(), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return from_cuda(e);
     }
     int sms = 152;
@@ -354,7 +447,7 @@ vktError build_plan(Plan& P, int32_t n, vktStructuredVolume* dst, vktStructuredV
     for (int l = 0; l < NL; ++l) {
         const int nl = loff[l + 1] - loff[l];
         if (nl == 0) continue;
-        BatchKernel kern = batch_kernel(KS[l / 4], (l / 2) % 2 == 1, l % 2 == 1);
+        BatchKernel kern = batch_kernel(KS[l / 6], (l / 2) % 3, l % 2 == 1);
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  static_cast<int>(lsmem[l]));
         if (e != cudaSuccess) return from_cuda(e);
@@ -409,8 +502,9 @@ vktError build_plan(Plan& P, int32_t n, vktStructuredVolume* dst, vktStructuredV
             if (nl == 0) continue;
             e = cudaStreamWaitEvent(side[l], fork, 0);
             if (e != cudaSuccess) break;
-            batch_kernel(KS[l / 4], (l / 2) % 2 == 1, l % 2 == 1)<<<lgrid[l], sep::NT, lsmem[l], side[l]>>>(
-                P.d_jobs, P.d_maps, P.d_items + loff[l], nl, P.d_counter + 32 * l, ctx.status);
+            batch_kernel(KS[l / 6], (l / 2) % 3, l % 2 == 1)<<<lgrid[l], sep::NT, lsmem[l], side[l]>>>(
+                P.d_jobs, P.d_maps, P.d_items + loff[l], nl, P.d_counter + 32 * l, ctx.status,
+                P.d_split);
             e = cudaGetLastError();
             if (e == cudaSuccess) e = cudaEventRecord(join[l], side[l]);
             ++kernels;
@@ -476,8 +570,8 @@ vktError build_plan(Plan& P, int32_t n, vktStructuredVolume* dst, vktStructuredV
                 per_sm_cap);
         for (int l = 0; l < NL; ++l)
             if (loff[l + 1] > loff[l])
-                fprintf(stderr, "[vkt]   k=%d%s%s: %d bricks, grid %d, smem %zu\n", KS[l / 4],
-                        (l / 2) % 2 ? " compensated" : "", l % 2 ? " narrow" : "",
+                fprintf(stderr, "[vkt]   k=%d%s%s: %d bricks, grid %d, smem %zu\n", KS[l / 6],
+                        (l / 2) % 3 == B_DOT2 ? " compensated" : (l / 2) % 3 == B_SPLIT ? " split" : "", l % 2 ? " narrow" : "",
                         loff[l + 1] - loff[l], lgrid[l], lsmem[l]);
     }
     return VKT_NO_ERROR;
@@ -538,7 +632,6 @@ extern "C" vktError vktApplyFilterBatchSV(int32_t n, vktStructuredVolume* dst, v
         put(key, src[i]->format);
         put(key, dst[i]->format);
         put(key, filters[i]->k);
-        put(key, s && separable_needs_comp(dst[i], src[i], filters[i]));
         const int shape[7] = {s ? 1 : 0, src[i]->dims[0], src[i]->dims[1], src[i]->dims[2],
                               static_cast<int>(src[i]->format) * 4 + static_cast<int>(dst[i]->format),
                               filters[i]->k, s && separable_needs_comp(dst[i], src[i], filters[i])};
@@ -556,6 +649,9 @@ extern "C" vktError vktApplyFilterBatchSV(int32_t n, vktStructuredVolume* dst, v
     }
     // current table contents (weights and epilogue constants of the separable volumes)
     std::vector<sep::Job> table(sep_idx.size());
+    std::vector<int> modes(sep_idx.size(), B_PLAIN);
+    std::vector<const Split*> splits(sep_idx.size(), nullptr);
+    std::list<Split> seen;
     for (size_t j = 0; j < sep_idx.size(); ++j) {
         const int i = sep_idx[j];
         const vktFilter_impl* f = filters[i];
@@ -568,7 +664,15 @@ extern "C" vktError vktApplyFilterBatchSV(int32_t n, vktStructuredVolume* dst, v
                 s3[a] += f->g[a][t];
             }
         epilogue_of(dst[i], src[i], s3[0] * s3[1] * s3[2], &J.a0, &J.a1, &J.qmax, &J.a0lo, &J.a1lo);
-        J.comp = separable_needs_comp(dst[i], src[i], f) ? 1 : 0;
+        J.sfmt = src[i]->format;
+        if (separable_needs_comp(dst[i], src[i], f)) {
+            modes[j] = B_DOT2;
+            if (src[i]->format == vktDataFormatUint16 && f->k >= 3) {
+                splits[j] = &split_of(seen, J, f->k);
+                if (splits[j]->ok) modes[j] = B_SPLIT;
+            }
+        }
+        put(key, modes[j]);
     }
 
     std::lock_guard<std::mutex> lock(g_plans_mutex);
@@ -604,7 +708,7 @@ extern "C" vktError vktApplyFilterBatchSV(int32_t n, vktStructuredVolume* dst, v
             for (int c = 0; c < NC && err == VKT_NO_ERROR; ++c) {
                 plans[c].key = key;
                 plans[c].device = dev;
-                err = build_plan(plans[c], n, dst, src, filters, sep_idx, dense_idx, force_dense,
+                err = build_plan(plans[c], n, dst, src, filters, sep_idx, dense_idx, modes, splits, force_dense,
                                  force_direct, ctx, cand[c].zchunk, cand[c].path & 15,
                                  (cand[c].path & 16) != 0);
             }
@@ -630,7 +734,7 @@ extern "C" vktError vktApplyFilterBatchSV(int32_t n, vktStructuredVolume* dst, v
         } else {
             P.key = key;
             P.device = dev;
-            err = build_plan(P, n, dst, src, filters, sep_idx, dense_idx, force_dense, force_direct,
+            err = build_plan(P, n, dst, src, filters, sep_idx, dense_idx, modes, splits, force_dense, force_direct,
                              ctx, tc.zchunk > 0 ? tc.zchunk : 64, std::max(0, tc.path) & 15,
                              (std::max(0, tc.path) & 16) != 0);
             if (err != VKT_NO_ERROR) {
@@ -664,6 +768,13 @@ extern "C" vktError vktApplyFilterBatchSV(int32_t n, vktStructuredVolume* dst, v
             J.a1lo = table[j].a1lo;
             cudaError_t e = cudaMemcpyAsync(P.d_jobs + j, &J, sizeof(sep::Job),
                                             cudaMemcpyHostToDevice, stream);
+            if (e != cudaSuccess) return from_cuda(e);
+        }
+        if (modes[j] == B_SPLIT &&
+            memcmp(P.split.data() + j * SPLIT_PITCH, splits[j]->w.data(), SPLIT_PITCH) != 0) {
+            memcpy(P.split.data() + j * SPLIT_PITCH, splits[j]->w.data(), SPLIT_PITCH);
+            cudaError_t e = cudaMemcpyAsync(P.d_split + j * SPLIT_PITCH, P.split.data() + j * SPLIT_PITCH,
+                                            SPLIT_PITCH, cudaMemcpyHostToDevice, stream);
             if (e != cudaSuccess) return from_cuda(e);
         }
     }
