@@ -181,6 +181,20 @@ VKT_API vktError vktStructuredVolumeCreateView(vktStructuredVolume* volume, void
                                        vktDataFormat format, float sx, float sy, float sz,
                                        float lo, float hi);
 
+/*
+ * n views in one call: view i covers dims[3 i] x dims[3 i + 1] x dims[3 i + 2] voxels at
+ * devPtrs[i]; format, cell size and range are the same for all.  Arguments and errors of
+ * vktStructuredVolumeCreateView for each of them; all n are created or none (volumes[] is then
+ * all NULL).  n >= 1.
+ */
+VKT_API vktError vktStructuredVolumeCreateViews(int32_t n, vktStructuredVolume* volumes,
+                                        void* const* devPtrs, const int32_t* dims,
+                                        vktDataFormat format, float sx, float sy, float sz,
+                                        float lo, float hi);
+
+/* vktStructuredVolumeDestroy for each of n volumes; the first error, if any, is returned. */
+VKT_API vktError vktStructuredVolumesDestroy(int32_t n, vktStructuredVolume* volumes);
+
 /* Releases the handle (and the device memory of an owning volume). */
 VKT_API vktError vktStructuredVolumeDestroy(vktStructuredVolume volume);
 

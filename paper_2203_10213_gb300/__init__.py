@@ -46,19 +46,27 @@ def build(force: bool = False) -> str:
     return _build.build(force=force)
 
 
+_torch_module = None
+_formats: dict = {}     # torch dtype -> format, filled with torch's import
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _formats.update({torch.uint8: U8, torch.float32: F32})
+        if hasattr(torch, "uint16"):
+            _formats[torch.uint16] = U16
+        _torch_module = torch
+    return _torch_module
 
 
 def _fmt_of_dtype(dtype) -> int:
-    torch = _torch()
-    table = {torch.uint8: U8, torch.float32: F32}
-    if hasattr(torch, "uint16"):
-        table[torch.uint16] = U16
-    if dtype not in table:
+    _torch()
+    fmt = _formats.get(dtype)
+    if fmt is None:
         raise TypeError(f"unsupported voxel dtype {dtype}")
-    return table[dtype]
+    return fmt
 
 
 def torch_dtype(fmt: int):
@@ -93,20 +101,42 @@ def set_policy(stream=None, path=None, debug=None, print_times=None) -> None:
     check(_lib.vktSetThreadExecutionPolicy(pol))
 
 
-@contextlib.contextmanager
-def policy(stream=None, path=None, debug=None, print_times=None):
-    """Temporarily sets the calling thread's execution policy (None: keep the setting)."""
-    old = get_policy()
-    set_policy(stream, path, debug, print_times)
-    try:
-        yield
-    finally:
-        check(_lib.vktSetThreadExecutionPolicy(old))
+class policy(contextlib.ContextDecorator):
+    """Temporarily sets the calling thread's execution policy (None: keep the setting).  The
+    policy is set, and put back, only where it differs from the thread's (a call on the thread's
+    own stream makes one library call here instead of four)."""
+
+    def __init__(self, stream=None, path=None, debug=None, print_times=None):
+        self._args = stream, path, debug, print_times
+
+    def _recreate_cm(self):
+        return policy(*self._args)
+
+    def __enter__(self):
+        stream, path, debug, print_times = self._args
+        old = get_policy()
+        new = (_stream_handle(stream),
+               old.path if path is None else PATHS[path] if isinstance(path, str) else int(path),
+               old.debug if debug is None else int(debug),
+               old.printTimes if print_times is None else int(bool(print_times)))
+        self._old = None
+        if new != (old.stream or 0, old.path, old.debug, old.printTimes):
+            check(_lib.vktSetThreadExecutionPolicy(
+                ExecutionPolicy(new[0], new[3], new[2], new[1])))
+            self._old = old
+
+    def __exit__(self, *exc):
+        if self._old is not None:
+            check(_lib.vktSetThreadExecutionPolicy(self._old))
+        return False
 
 
 def _stream_handle(stream) -> int:
     if stream is None:
         torch = _torch()
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if torch.cuda.is_initialized() and raw is not None:
+            return int(raw(torch.cuda.current_device()))     # current_stream() takes 3 us
         return int(torch.cuda.current_stream().cuda_stream) if torch.cuda.is_available() else 0
     if isinstance(stream, int):
         return stream
@@ -219,6 +249,35 @@ class StructuredVolume:
             self.destroy()
         except Exception:
             pass
+
+
+class _Views:
+    """Views of several tensors (or of the volumes of one batch tensor) for one library call, made
+    and destroyed by one call each.  `array` is the handle array; the tensors are kept alive."""
+
+    def __init__(self, pointers, dims, fmt: int, lo: float = 0.0, hi: float = 1.0, keep=None):
+        n = self.n = len(pointers)
+        self.array, self.keep = (ctypes.c_void_p * n)(), keep
+        check(_lib.vktStructuredVolumeCreateViews(n, self.array, (ctypes.c_void_p * n)(*pointers),
+                                                  (ctypes.c_int32 * (3 * n))(*dims), fmt, 1.0, 1.0, 1.0,
+                                                  lo, hi), "vktStructuredVolumeCreateViews")
+
+    @classmethod
+    def of_batch(cls, t):
+        """The volumes t[0], t[1], ... of a contiguous (n, nz, ny, nx) CUDA tensor."""
+        if t.dim() != 4 or not t.is_contiguous() or not t.is_cuda:
+            raise ValueError("batch tensors are contiguous CUDA tensors of shape (n, nz, ny, nx)")
+        n, nz, ny, nx = t.shape
+        step = nz * ny * nx * t.element_size()
+        base = t.data_ptr()
+        return cls([base + b * step for b in range(n)], (nx, ny, nz) * n, _fmt_of_dtype(t.dtype), keep=t)
+
+    def __enter__(self):
+        return self.array
+
+    def __exit__(self, *exc):
+        check(_lib.vktStructuredVolumesDestroy(self.n, self.array))
+        return False
 
 
 # ------------------------------------------------------------------ filters
@@ -379,19 +438,20 @@ def brick_decompose(src_t, brick, ghost: int = 0, src_range=(0.0, 1.0), stream=N
     cx, cy, cz = brick_counts(src, brick)
     nz, ny, nx = src_t.shape
     bx, by, bz = map(int, brick)
-    tensors, views = [], []
-    for kz in range(cz):
-        for ky in range(cy):
-            for kx in range(cx):
-                shape = (min(bz, nz - kz * bz) + 2 * ghost, min(by, ny - ky * by) + 2 * ghost,
-                         min(bx, nx - kx * bx) + 2 * ghost)
-                t = torch.empty(shape, dtype=src_t.dtype, device=src_t.device)
+    grow = 2 * ghost
+    sizes = [[min(s, n - i * s) + grow for i in range(c)] for s, n, c in ((bx, nx, cx), (by, ny, cy), (bz, nz, cz))]
+    tensors, pointers, dims = [], [], []
+    for dz in sizes[2]:
+        for dy in sizes[1]:
+            for dx in sizes[0]:
+                t = torch.empty((dz, dy, dx), dtype=src_t.dtype, device=src_t.device)
                 tensors.append(t)
-                views.append(StructuredVolume.from_tensor(t, *src_range))
-    arr = (ctypes.c_void_p * len(views))(*(v.handle.value for v in views))
-    with policy(stream=stream):
-        check(_lib.vktBrickDecomposeSV(arr, len(views), src.handle, bx, by, bz, int(ghost)),
-              "vktBrickDecomposeSV")
+                pointers.append(t.data_ptr())
+                dims += (int(dx), int(dy), int(dz))
+    with _Views(pointers, dims, _fmt_of_dtype(src_t.dtype), *src_range, keep=tensors) as views:
+        with policy(stream=stream):
+            check(_lib.vktBrickDecomposeSV(views, len(tensors), src.handle, bx, by, bz, int(ghost)),
+                  "vktBrickDecomposeSV")
     return tensors
 
 
@@ -475,10 +535,10 @@ def _autograd_function():
             w_host = w.detach().float().cpu().numpy()
             filt = Filter.dense(w_host)
             y = torch.empty_like(xb)
-            vx = [StructuredVolume.from_tensor(xb[b]) for b in range(xb.shape[0])]
-            vy = [StructuredVolume.from_tensor(y[b]) for b in range(xb.shape[0])]
-            with policy(path=path):
-                apply_filter_batch(vy, vx, [filt] * len(vx))
+            n = xb.shape[0]
+            with _Views.of_batch(xb) as vx, _Views.of_batch(y) as vy, policy(path=path):
+                check(_lib.vktApplyFilterBatchSV(n, vy, vx, (ctypes.c_void_p * n)(*[filt.handle.value] * n)),
+                      "vktApplyFilterBatchSV")
             ctx.save_for_backward(xb)
             ctx.filt = filt
             ctx.w_shape = w.shape
@@ -496,10 +556,14 @@ def _autograd_function():
                 k3 *= d
             gw = torch.empty(k3, dtype=torch.float32, device=xb.device) if need_w else None
             n = xb.shape[0]
-            apply_filter_backward_batch(
-                [StructuredVolume.from_tensor(gx[b]) for b in range(n)] if need_x else None, gw,
-                [StructuredVolume.from_tensor(gyb[b]) for b in range(n)],
-                [StructuredVolume.from_tensor(xb[b]) for b in range(n)], ctx.filt)
+            with _Views.of_batch(xb) as vx, _Views.of_batch(gyb) as vgy, policy():
+                args = (ctypes.c_void_p(gw.data_ptr()) if need_w else None, vgy, vx, ctx.filt.handle)
+                if need_x:
+                    with _Views.of_batch(gx) as vgx:
+                        err = _lib.vktApplyFilterBackwardBatchSV(n, vgx, *args)
+                else:
+                    err = _lib.vktApplyFilterBackwardBatchSV(n, None, *args)
+                check(err, "vktApplyFilterBackwardBatchSV")
             return ((gx.reshape(ctx.shape) if need_x else None),
                     (gw.reshape(ctx.w_shape) if need_w else None), None)
 

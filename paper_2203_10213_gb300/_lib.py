@@ -36,6 +36,9 @@ SIGNATURES = {
     "vktStructuredVolumeCreate": [ctypes.POINTER(p), i32, i32, i32, c_err, f32, f32, f32, f32, f32],
     "vktStructuredVolumeCreateView": [ctypes.POINTER(p), p, i32, i32, i32, c_err, f32, f32, f32,
                                       f32, f32],
+    "vktStructuredVolumeCreateViews": [i32, ctypes.POINTER(p), ctypes.POINTER(p), pi32, c_err, f32, f32,
+                                       f32, f32, f32],
+    "vktStructuredVolumesDestroy": [i32, ctypes.POINTER(p)],
     "vktStructuredVolumeDestroy": [p],
     "vktStructuredVolumeGetDims": [p, pi32, pi32, pi32],
     "vktStructuredVolumeGetDataFormat": [p, ctypes.POINTER(c_err)],

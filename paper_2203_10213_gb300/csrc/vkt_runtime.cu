@@ -496,6 +496,37 @@ vktError vktStructuredVolumeCreateView(vktStructuredVolume* volume, void* devPtr
     return create_volume(volume, devPtr, 0, dx, dy, dz, format, sx, sy, sz, lo, hi);
 }
 
+vktError vktStructuredVolumeCreateViews(int32_t n, vktStructuredVolume* volumes, void* const* devPtrs,
+                                        const int32_t* dims, vktDataFormat format, float sx,
+                                        float sy, float sz, float lo, float hi)
+{
+    if (n < 1 || !volumes) return VKT_ERROR_INVALID_VALUE;
+    for (int32_t i = 0; i < n; ++i) volumes[i] = nullptr;
+    if (!devPtrs || !dims) return VKT_ERROR_INVALID_VALUE;
+    for (int32_t i = 0; i < n; ++i) {
+        const vktError err = create_volume(&volumes[i], devPtrs[i], 0, dims[3 * i], dims[3 * i + 1],
+                                           dims[3 * i + 2], format, sx, sy, sz, lo, hi);
+        if (err == VKT_NO_ERROR) continue;
+        for (int32_t j = 0; j < i; ++j) {
+            vktStructuredVolumeDestroy(volumes[j]);
+            volumes[j] = nullptr;
+        }
+        return err;
+    }
+    return VKT_NO_ERROR;
+}
+
+vktError vktStructuredVolumesDestroy(int32_t n, vktStructuredVolume* volumes)
+{
+    if (n < 1 || !volumes) return VKT_ERROR_INVALID_VALUE;
+    vktError first = VKT_NO_ERROR;
+    for (int32_t i = 0; i < n; ++i) {
+        const vktError err = vktStructuredVolumeDestroy(volumes[i]);
+        if (first == VKT_NO_ERROR) first = err;
+    }
+    return first;
+}
+
 vktError vktStructuredVolumeDestroy(vktStructuredVolume volume)
 {
     if (!valid(volume)) return VKT_ERROR_INVALID_HANDLE;
