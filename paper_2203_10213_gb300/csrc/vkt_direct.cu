@@ -7,6 +7,11 @@ namespace vkt {
 
 vktError launch_direct(const Job& job, const float* w, int k, const Ctx& ctx)
 {
+    if (k == 3) {
+        bool taken = false;
+        const vktError err = launch_star(job, w, ctx, &taken);
+        if (taken) return err;
+    }
     if (job.comp) return launch_direct_comp(job, w, k, ctx);
     switch (k) {
     case 1: return dir::launch_k<1, false>(job, w, ctx);

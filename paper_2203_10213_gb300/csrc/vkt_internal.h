@@ -179,6 +179,8 @@ vktError prepare_kernel(const Ctx& ctx, const void* kern, int threads, size_t sm
 // the compensated kernels when job.comp is set (launch_direct_comp).
 vktError launch_direct(const Job& job, const float* w, int k, const Ctx& ctx);
 vktError launch_direct_comp(const Job& job, const float* w, int k, const Ctx& ctx);
+// 3^3 filters with taps on the axes only, on integer volumes (*taken: the job is one).
+vktError launch_star(const Job& job, const float* w, const Ctx& ctx, bool* taken);
 // The listed modes of the compensated direct kernel, where they suit the job (*taken).
 struct ListPlan;
 vktError launch_direct_listed(const Job& job, const float* w, int k, const Ctx& ctx, bool* taken);
