@@ -289,6 +289,7 @@ __device__ __forceinline__ void direct_body(const CUtensorMap& tmap, const Direc
     const int ox = x0 + tx * RX;
     const int nvalid = (ROI ? p.sx1 : p.nx) - ox;
     const int first = (ROI && p.sx0 > ox) ? p.sx0 - ox : 0;   // leading columns outside the region
+    const int nwide = wide_count(dst, nvalid);
     const int yend = ROI ? p.sy1 : p.ny;
     bool failed = false;
 
@@ -555,7 +556,7 @@ __device__ __forceinline__ void direct_body(const CUtensorMap& tmap, const Direc
                 for (int x = 0; x < RX; ++x) row[x] = lane(sl0, i, x);
                 if (oy < yend && nvalid > 0) {
                     const int64_t idx = (static_cast<int64_t>(oz) * p.ny + oy) * p.nx + ox;
-                    store_row<RX>(dst, dfmt, idx, nvalid, row, p.a0, p.a1, p.qmax, first);
+                    store_row<RX>(dst, dfmt, idx, nvalid, row, p.a0, p.a1, p.qmax, first, nwide);
                 }
             }
         }

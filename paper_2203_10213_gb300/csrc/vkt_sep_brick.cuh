@@ -247,6 +247,7 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
     const int ox = x0 + tx * RX;
     const int nvalid = (ROI ? J.sx1 : J.nx) - ox;
     const int first = (ROI && J.sx0 > ox) ? J.sx0 - ox : 0;   // leading columns outside the region
+    const int nwide = wide_count(J.dst, nvalid);
     const int yend = ROI ? J.sy1 : J.ny;
     bool failed = false;
 
@@ -411,7 +412,7 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
             const int oy = y0 + ty * RY + i;
             if (it >= 2 * R && oy < yend && nvalid > 0) {
                 const int64_t idx = (static_cast<int64_t>(pfirst + it - R) * J.ny + oy) * J.nx + ox;
-                store_row<RX>(J.dst, dfmt, idx, nvalid, rowv, J.a0, J.a1, J.qmax, first);
+                store_row<RX>(J.dst, dfmt, idx, nvalid, rowv, J.a0, J.a1, J.qmax, first, nwide);
             }
         };
         if constexpr (PAIR) {

@@ -506,21 +506,28 @@ __device__ __forceinline__ void store_codes(void* dst, int dfmt, int64_t idx, in
     }
 }
 
+// How many results of a row may be stored as one: those of a float32 destination that starts on a
+// 16-byte boundary (store_row then needs to look at the row's own offset only).
+__device__ __forceinline__ int wide_count(const void* dst, int nvalid)
+{
+    return (reinterpret_cast<uintptr_t>(dst) & 15) == 0 ? nvalid : 0;
+}
+
 // Writes results first .. nvalid-1 of RX consecutive results of one row (from idx), mapped
-// to the destination format.
+// to the destination format; nwide: wide_count(dst, nvalid).
 template <int RX>
 __device__ __forceinline__ void store_row(void* dst, int dfmt, int64_t idx, int nvalid,
                                           const float (&acc)[RX], float a0, float a1, float qmax,
-                                          int first = 0)
+                                          int first, int nwide)
 {
     float v[RX];
 #pragma unroll
     for (int x = 0; x < RX; ++x) v[x] = fmaf(a1, acc[x], a0);
     if (dfmt == FMT_F32) {
         float* d = reinterpret_cast<float*>(dst) + idx;
-        if (RX == 4 && first == 0 && nvalid >= 4 && (idx & 3) == 0) {
+        if (RX == 4 && first == 0 && nwide >= 4 && (idx & 3) == 0) {
             *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
-        } else if (RX == 2 && first == 0 && nvalid >= 2 && (idx & 1) == 0) {
+        } else if (RX == 2 && first == 0 && nwide >= 2 && (idx & 1) == 0) {
             *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
         } else {
 #pragma unroll
