@@ -115,11 +115,12 @@ __host__ __device__ constexpr size_t smem_bytes(int sfmt, bool rows = false)
            static_cast<size_t>(Geo::FH) * tile_x<BXG>() * sizeof(float);  // x-pass output
 }
 
-// row copies of a plane, by the way the kernel uses
-template <typename Geo, bool BULK, typename... A>
+// row copies of a plane: as bulk copies in the batch, for float32 sources and where the format
+// (SF) is chosen at run time, else as 16-byte blocks
+template <typename Geo, bool BULK, int SF, typename... A>
 __device__ __forceinline__ void copy_rows(A... a)
 {
-    if constexpr (BULK)
+    if constexpr (BULK || SF < 0 || SF == FMT_F32)
         issue_rows_bulk<Geo, NT>(a...);
     else
         issue_rows<Geo, NT>(a...);
@@ -211,7 +212,7 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
     } else if (rows) {
         for (int s = 0; s < NS && s < nplanes; ++s) {
             const uint32_t q = g0 + s;
-            copy_rows<Geo, BULK>(raw + (q % NS) * rawb, &bars[q % NS], J.src, vol_bytes,
+            copy_rows<Geo, BULK, SF>(raw + (q % NS) * rawb, &bars[q % NS], J.src, vol_bytes,
                                 sfmt, J.nx, J.ny, J.nz, x0, y0, pfirst + s, tid);
         }
         __syncthreads();   // every thread's expect_tx precedes the single arrival
@@ -342,7 +343,7 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
                 ++issued;
             } else if (rows && it + NS < nplanes) {
                 // all threads; the arrival follows the next plane's barrier
-                copy_rows<Geo, BULK>(raw + s * rawb, &bars[s], J.src, vol_bytes, sfmt, J.nx, J.ny,
+                copy_rows<Geo, BULK, SF>(raw + s * rawb, &bars[s], J.src, vol_bytes, sfmt, J.nx, J.ny,
                                     J.nz, x0, y0, pfirst + it + NS, tid);
                 pend = s;
             }
@@ -374,7 +375,7 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
             ++issued;
         } else if (rows && it + NS < nplanes) {
             // all threads; the arrival follows the x-pass barrier below
-            copy_rows<Geo, BULK>(raw + s * rawb, &bars[s], J.src, vol_bytes, sfmt, J.nx, J.ny,
+            copy_rows<Geo, BULK, SF>(raw + s * rawb, &bars[s], J.src, vol_bytes, sfmt, J.nx, J.ny,
                                 J.nz, x0, y0, pfirst + it + NS, tid);
         }
         // x pass: T1[row][x] = sum_a gx[a] F[row][x + a], 4 outputs per item
@@ -612,7 +613,7 @@ __device__ __forceinline__ bool brick_comp(const Job& J, const Wt& G, const CUte
     } else if (rows) {
         for (int s = 0; s < STAGES && s < nplanes; ++s) {
             const uint32_t q = g0 + s;
-            copy_rows<Geo, BULK>(raw + (q % STAGES) * rawb, &bars[q % STAGES], J.src, vol_bytes,
+            copy_rows<Geo, BULK, -1>(raw + (q % STAGES) * rawb, &bars[q % STAGES], J.src, vol_bytes,
                                 J.sfmt, J.nx, J.ny, J.nz, x0, y0, pfirst + s, tid);
         }
         __syncthreads();   // every thread's expect_tx precedes the single arrival
@@ -667,7 +668,7 @@ __device__ __forceinline__ bool brick_comp(const Job& J, const Wt& G, const CUte
             ++issued;
         } else if (rows && it + STAGES < nplanes) {
             // all threads; the arrival follows the x-pass barrier below
-            copy_rows<Geo, BULK>(raw + s * rawb, &bars[s], J.src, vol_bytes, J.sfmt, J.nx, J.ny,
+            copy_rows<Geo, BULK, -1>(raw + s * rawb, &bars[s], J.src, vol_bytes, J.sfmt, J.nx, J.ny,
                                 J.nz, x0, y0, pfirst + it + STAGES, tid);
         }
         // x pass (inputs exact): T1[row][x] = Dot2(gx, F[row][x .. x+k-1])

@@ -243,7 +243,7 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
     } else if (rows) {
         for (int s = 0; s < STAGES && s < nplanes; ++s) {
             const uint32_t q = g0 + s;
-            copy_rows<Geo, BULK>(raw + (q % STAGES) * rawb, &bars[q % STAGES], J.src, vol_bytes, SF,
+            copy_rows<Geo, BULK, SF>(raw + (q % STAGES) * rawb, &bars[q % STAGES], J.src, vol_bytes, SF,
                                 J.nx, J.ny, J.nz, x0, y0, pfirst + s, tid);
         }
         __syncthreads();   // every thread's expect_tx precedes the single arrival
@@ -368,7 +368,7 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
             ++issued;
         } else if (rows && it + STAGES < nplanes) {
             // all threads; the arrival follows the next plane's wait
-            copy_rows<Geo, BULK>(raw + s * rawb, &bars[s], J.src, vol_bytes, SF, J.nx, J.ny, J.nz, x0,
+            copy_rows<Geo, BULK, SF>(raw + s * rawb, &bars[s], J.src, vol_bytes, SF, J.nx, J.ny, J.nz, x0,
                                 y0, pfirst + it + STAGES, tid);
             pend = s;
         }

@@ -101,8 +101,8 @@ __global__ void __launch_bounds__(NT, 2)
             w[0] = t.x;
             w[1] = t.y;
         }
-        v[0] = make_float2(code_float<SF, CENTRE>(w, 0), code_float<SF, CENTRE>(w, 1));
-        v[1] = make_float2(code_float<SF, CENTRE>(w, 2), code_float<SF, CENTRE>(w, 3));
+        v[0] = code_pair<SF, CENTRE>(w, 0);
+        v[1] = code_pair<SF, CENTRE>(w, 2);
     };
     auto load1 = [&](const unsigned char* q) {
         const uint32_t c = SF == FMT_U8 ? *q : *reinterpret_cast<const uint16_t*>(q);
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(NT, 2)
         // the plane before this one: its stage is free once the slowest warp has read it
         const int refill = it - 1 + STAGES;
         if (tid == 0 && it >= 1 && refill < nplanes) {
-            // (a refill that is not made ends the march at the wait for its plane)
+            // (a refill that is not made ends every warp's march at the wait for its plane)
             if (ok && mbar_wait(&empty[refill % STAGES], ((it - 1) / STAGES) & 1))
                 issue(refill);
             else

@@ -207,9 +207,11 @@ struct Brick {
 // issue_rows, so the phase cannot complete before all copies are counted, and the
 // plain-loaded bytes are visible to whoever waits on the phase.
 // (One bulk copy per row, issue_rows_bulk, makes the kernels wait for the copy unit, which takes
-// these 112-byte copies one at a time: 302^3 uint8, k = 5, into uint8 97 us against 88, into float32
-// 87 against 78.  The batch, with several kernels' bricks on an SM, has work for that time and
-// spends fewer instructions with it: 570 against 584 us for 128 mixed volumes.)
+// these 112-byte copies one at a time: 302^3 uint8, k = 5, separable into uint8 97 us against 88, into
+// float32 82 against 73, direct 180 against 167.  It stays where it is the faster one: float32
+// sources, whose rows are three times as many blocks (k = 3 66 against 75 us), kernels with the
+// format chosen at run time (direct k = 3 uint16 into float32 95 against 120), and the batch, where
+// other kernels' bricks on the SM have work for that time (570 against 584 us for 128 mixed volumes).)
 __device__ __forceinline__ uint32_t row_shift_elems(uint32_t zterm, int gy, int nx, int x0, int xa,
                                                     int fmt)
 {

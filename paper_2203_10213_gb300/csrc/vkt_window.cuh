@@ -11,19 +11,25 @@
 
 namespace vkt {
 
-// code i of the packed words w as a float, minus 2^(bits-1) if CENTRE (exact): 2^23 + code is
-// built by a byte permute, then one subtraction
-template <int SF, bool CENTRE>
-__device__ __forceinline__ float code_float(const uint32_t* w, int i)
+// 2^23 + code i of the packed words w, as a float's bits (exact), by a byte permute
+template <int SF>
+__device__ __forceinline__ uint32_t code_bits(const uint32_t* w, int i)
 {
     static_assert(SF == FMT_U8 || SF == FMT_U16, "integer sources");
-    if constexpr (SF == FMT_U8) {
-        const uint32_t b = __byte_perm(w[i >> 2], 0x4B000000u, 0x7440u + (i & 3));
-        return __uint_as_float(b) - (CENTRE ? 8388608.f + 128.f : 8388608.f);
-    } else {
-        const uint32_t b = __byte_perm(w[i >> 1], 0x4B000000u, (i & 1) ? 0x7432u : 0x7410u);
-        return __uint_as_float(b) - (CENTRE ? 8388608.f + 32768.f : 8388608.f);
-    }
+    if constexpr (SF == FMT_U8)
+        return __byte_perm(w[i >> 2], 0x4B000000u, 0x7440u + (i & 3));
+    else
+        return __byte_perm(w[i >> 1], 0x4B000000u, (i & 1) ? 0x7432u : 0x7410u);
+}
+
+// codes i and i + 1 as floats, minus 2^(bits-1) if CENTRE (exact): the offset of both is taken off by
+// one packed addition
+template <int SF, bool CENTRE>
+__device__ __forceinline__ float2 code_pair(const uint32_t* w, int i)
+{
+    constexpr float off = CENTRE ? 8388608.f + (SF == FMT_U8 ? 128.f : 32768.f) : 8388608.f;
+    return __fadd2_rn(make_float2(__uint_as_float(code_bits<SF>(w, i)), __uint_as_float(code_bits<SF>(w, i + 1))),
+                      make_float2(-off, -off));
 }
 
 // win[e] = code at raw column col + shift + e of the stage row at `row`, e < K + 3.  FIXED:
@@ -45,7 +51,11 @@ __device__ __forceinline__ void window(const unsigned char* row, int col, uint32
 #pragma unroll
         for (int i = 0; i < NW; ++i) w[i] = p[i];
 #pragma unroll
-        for (int e = 0; e < K + 3; ++e) win[e] = code_float<SF, CENTRE>(w, O / ES + e);
+        for (int e = 0; e < K + 3; e += 2) {
+            const float2 v = code_pair<SF, CENTRE>(w, O / ES + e);
+            win[e] = v.x;
+            win[e + 1] = v.y;
+        }
     } else {
         constexpr int NW = ((K + 3) * ES + 3) / 4;
         const uint32_t at = (static_cast<uint32_t>(col) + shift) * ES;
@@ -57,7 +67,11 @@ __device__ __forceinline__ void window(const unsigned char* row, int col, uint32
 #pragma unroll
         for (int i = 0; i < NW; ++i) w[i] = __funnelshift_r(w[i], w[i + 1], bits);
 #pragma unroll
-        for (int e = 0; e < K + 3; ++e) win[e] = code_float<SF, CENTRE>(w, e);
+        for (int e = 0; e < K + 3; e += 2) {
+            const float2 v = code_pair<SF, CENTRE>(w, e);
+            win[e] = v.x;
+            win[e + 1] = v.y;
+        }
     }
 }
 
