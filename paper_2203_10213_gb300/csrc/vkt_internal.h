@@ -206,6 +206,12 @@ vktError reduce_weight_grad(const float* partials, size_t nspatial, int k, float
 vktError launch_separable(const Job& job, const float* gx, const float* gy, const float* gz,
                           int k, const Ctx& ctx);
 
+// The walking separable kernels (vkt_walk.cuh); *taken: the job is one of theirs.
+vktError launch_walk_k3(const Job& job, const float* gx, const float* gy, const float* gz, const Ctx& ctx,
+                        bool* taken);
+vktError launch_walk_k5(const Job& job, const float* gx, const float* gy, const float* gz, const Ctx& ctx,
+                        bool* taken);
+
 // Tensor-core path: VKT_NO_ERROR if it can evaluate this triple, else why not.
 vktError tensor_available(const vktStructuredVolume_impl* dst, const vktStructuredVolume_impl* src,
                           const vktFilter_impl* f);

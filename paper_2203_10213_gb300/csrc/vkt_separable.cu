@@ -19,6 +19,12 @@ vktError launch_separable_k3(const Job& job, const float* gx, const float* gy, c
 vktError launch_separable(const Job& job, const float* gx, const float* gy, const float* gz,
                           int k, const Ctx& ctx)
 {
+    if (k == 3 || k == 5) {
+        bool taken = false;
+        const vktError err = k == 3 ? launch_walk_k3(job, gx, gy, gz, ctx, &taken)
+                                    : launch_walk_k5(job, gx, gy, gz, ctx, &taken);
+        if (taken) return err;
+    }
     switch (k) {
     case 1: return launch_separable_k1(job, gx, gy, gz, ctx);
     case 3: return launch_separable_k3(job, gx, gy, gz, ctx);
