@@ -9,7 +9,9 @@ vktError launch_direct(const Job& job, const float* w, int k, const Ctx& ctx)
 {
     if (k == 3) {
         bool taken = false;
-        const vktError err = launch_star(job, w, ctx, &taken);
+        vktError err = launch_star(job, w, ctx, &taken);
+        if (taken) return err;
+        err = launch_march3(job, w, ctx, &taken);
         if (taken) return err;
     }
     if (job.comp) return launch_direct_comp(job, w, k, ctx);

@@ -181,6 +181,8 @@ vktError launch_direct(const Job& job, const float* w, int k, const Ctx& ctx);
 vktError launch_direct_comp(const Job& job, const float* w, int k, const Ctx& ctx);
 // 3^3 filters with taps on the axes only, on integer volumes (*taken: the job is one).
 vktError launch_star(const Job& job, const float* w, const Ctx& ctx, bool* taken);
+// Dense 3^3 filters of float32 volumes, marching through the raw stages (*taken: the job is one).
+vktError launch_march3(const Job& job, const float* w, const Ctx& ctx, bool* taken);
 // The listed modes of the compensated direct kernel, where they suit the job (*taken).
 struct ListPlan;
 vktError launch_direct_listed(const Job& job, const float* w, int k, const Ctx& ctx, bool* taken);

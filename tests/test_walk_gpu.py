@@ -1,5 +1,6 @@
-"""The kernel that marches through the raw stages (separable: vkt_walk.cuh): bit-identical to the general kernel, which a call with a region of interest takes,
-at tile edges, and which calls it takes."""
+"""The kernels that march through the raw stages (separable: vkt_walk.cuh, dense 3^3 of float32:
+vkt_march3.cu): bit-identical to the general kernels, which a call with a region of interest takes,
+at tile edges, and which calls they take."""
 import os
 import sys
 
@@ -67,12 +68,37 @@ def test_separable_codes(src, capfd):
             "separable-walk", capfd, 20)
 
 
+@pytest.mark.parametrize("shape", [(133, 305, 256), (200, 385, 260 - 68), (200, 401, 132 + 224)])
+def test_dense_float32(shape, capfd):
+    r = np.random.RandomState(6)
+    filt = vkt.Filter.dense(r.uniform(-1, 1, (3, 3, 3)).astype(np.float32))
+    compare(source(shape, torch.float32, 5), filt, torch.float32, "direct", "direct-march", capfd, 2 * 27)
+
+
+def test_dense_float32_batch(capfd):
+    # volumes of one allocation are one launch; each has its own faces
+    src = source((4, 72, 272, 128), torch.float32, 7)
+    w = np.random.RandomState(8).uniform(-1, 1, (3, 3, 3)).astype(np.float32)
+    capfd.readouterr()
+    with vkt.policy(debug=vkt.DEBUG_LOG):
+        out = vkt.apply_filter_autograd(torch.from_numpy(src).cuda(), torch.from_numpy(w).cuda(), "direct")
+    torch.cuda.synchronize()
+    vkt.synchronize()
+    assert "direct-march" in capfd.readouterr().err
+    for i in range(4):
+        np.testing.assert_array_equal(out[i].cpu().numpy(),
+                                      run(src[i], vkt.Filter.dense(w), torch.float32, path="direct"))
+
+
 def test_which_calls_take_it(capfd):
+    dense = vkt.Filter.dense(np.random.RandomState(9).uniform(-1, 1, (3, 3, 3)).astype(np.float32))
     gauss = vkt.Filter.gaussian(3, 1.0)
     for shape, src, filt, path in (((9, 20, 32), torch.float32, gauss, "separable"),
                                    ((9, 20, 38), torch.float32, gauss, "separable"),
-                                   ((9, 20, 256), torch.uint8, gauss, "separable")):
+                                   ((9, 20, 256), torch.uint8, gauss, "separable"),
+                                   ((9, 20, 128), torch.float32, dense, "direct"),
+                                   ((133, 305, 144), torch.float32, dense, "direct")):
         capfd.readouterr()
         run(source(shape, src, 1), filt, torch.float32, path=path)
         err = capfd.readouterr().err
-        assert "separable-walk" not in err
+        assert "separable-walk" not in err and "direct-march" not in err
