@@ -18,11 +18,20 @@
 // The items of a launch may span nvol volumes of equal dims (a training batch): one 128^3 volume
 // has too few of them to give every SM one, eight have.
 //
-// Warp roles (448 threads, one CTA per SM, persistent over (x, y, z-chunk) work items):
-//   warp 0       TMEM allocation; lane 0 issues TMA loads of f32 plane tiles
-//   warp 1       lane 0 issues the MMAs and commits
-//   warps 2..5   convert a plane tile to fp16 hi/lo operands (clamp-to-edge, scale)
-//   warps 6..13  epilogue: TMEM -> registers, z-march accumulate, store
+// Warp roles (640 threads, one CTA per SM, persistent over (x, y, z-chunk) work items):
+//   warp 1         lane 0 issues the MMAs and commits
+//   warp 5         lane 0 issues TMA loads of f32 plane tiles
+//   warps 4g+0, 2, 3 (g < 3)   convert plane tiles to fp16 hi/lo operands (clamp-to-edge, scale)
+//   warps 12..19   epilogue: TMEM -> registers, z-march accumulate, store
+// What bounds it: an MMA of 128 x 64 x 16 reads 6 KB of shared memory, 48 of its 55 cycles, and a
+// plane of an item at k = 7 has 42 of them (2290 cycles of the 2980 it takes; the rest is the hand-off
+// between planes and the epilogue's and converters' share of shared memory).  Two things kept the
+// MMAs from that rate.  (1) Warps 1, 5, 9, ... share a scheduler: with converters among them an MMA took
+// 70 to 80 cycles to issue.  (2) A converter's loads and stores wait for shared memory behind the
+// MMAs, a plane takes a group 5800 cycles, so two operand buffers (and one group) ran dry; hence three
+// groups with a buffer each, and the registers moved from them to the epilogue (setmaxnreg).
+// 1024 x 1024 x 256, before and after: k = 5 1413 / 1087 us, k = 7 1655 / 1413, k = 9 2063 / 1752; 128^3, k = 7
+// 68 / 33.  No gain from: A operands on whole 128-byte lines, collector reuse of A, a second D.
 // Every wait is bounded; on a timeout the CTA records it, drains what it issued and exits.
 #include <cuda_fp16.h>
 
@@ -39,10 +48,16 @@ namespace {
 constexpr int MROWS = 128;                 // output rows per tile (MMA M)
 constexpr int XT = 2;                      // x tiles of 8 outputs per work item
 constexpr int NCH = XT + 1;                // 8-wide input chunks per plane tile
-constexpr int STAGES = 4;
-constexpr int NTHREADS = 448;
-constexpr int CONV_WARP0 = 2, NCONV = 128;
-constexpr int EPI_WARP0 = 6, NEPI = 256;
+constexpr int STAGES = 5;
+constexpr int CGRP = 3;                    // converter groups, one per operand buffer
+constexpr int CONV_WARPS = NCH, NCONV = CONV_WARPS * 32;   // of a group: a warp per chunk
+constexpr int MMA_WARP = 1, TMA_WARP = 5, EPI_WARP0 = 12, NEPI = 256;
+constexpr int NTHREADS = EPI_WARP0 * 32 + NEPI;
+static_assert(CONV_WARPS == 3 && EPI_WARP0 == 4 * CGRP, "three of every four warps convert");
+// Registers of a thread at launch, then of the first three warpgroups and of the epilogue's two
+// (k = 7 80 and 120: 1417 us, 72 and 128: 1514, where the converters spill, 88 and 104: 1413).
+constexpr int REGS = 96, REGS_CONV = 88, REGS_EPI = 104;
+static_assert(3 * REGS_CONV + 2 * REGS_EPI <= 5 * REGS && NTHREADS == 5 * 128, "shares of the launch's registers");
 constexpr int SC_RING = 8;
 
 template <int K>
@@ -51,28 +66,25 @@ struct TcCfg {
     static constexpr int ROWS = MROWS + 2 * R;            // input rows of a plane tile
     static constexpr int SLOTS = ((K + 1) / 2) * 2;       // even, so N is a multiple of 16
     static constexpr int N = SLOTS * 8;
-    // CAT: the hi*hi and hi*lo products share one MMA of width 2N over the stacked
-    // operand [T_hi | T_lo], so A_hi is read once per (dy, x tile); the D columns [0,N)
-    // then hold hi*hi + lo*hi and [N,2N) hold hi*lo.  Measured slower on GB300 (the
-    // epilogue reads twice the columns), so it is off.
-    static constexpr bool CAT = false;
-    static constexpr int DN = CAT ? 2 * N : N;          // TMEM columns per (buffer, x tile)
+    static constexpr int DN = N;                         // TMEM columns per (buffer, x tile)
     static constexpr int DBUF = 3;                       // TMEM accumulator buffers
     static_assert(DBUF * XT * DN <= 512, "TMEM holds 512 columns");
     static constexpr int TMEM_COLS = (DBUF * XT * DN <= 256) ? 256 : 512;
     static constexpr int STAGE_BYTES = ((ROWS * NCH * 8 * 4) + 1023) & ~1023;
     static constexpr int STAGE_TX = ROWS * NCH * 8 * 4;
-    static constexpr int OP_BYTES = ((NCH * ROWS * 16) + 1023) & ~1023;   // one fp16 plane
+    // an operand plane: per 8-wide chunk, ROWS rows of 16 bytes (an A operand shifted down by b rows
+    // starts 16 b bytes further on)
+    static constexpr int CHUNK_BYTES = ROWS * 16;
+    static constexpr int OP_BYTES = (NCH * CHUNK_BYTES + 1023) & ~1023;   // one fp16 plane
     static constexpr int B_BYTES = 2 * N * 16;                            // one Toeplitz (hi or lo)
-    // converter items: (chunk, row, half) with the half fastest, 4 values each, so that a
-    // quarter warp's 16-byte reads of the stage (rows 96 bytes apart) and its 8-byte writes
-    // of the operand planes touch distinct banks
-    static constexpr int UNITS = NCH * ROWS * 2;
-    static constexpr int UPT = (UNITS + NCONV - 1) / NCONV;               // items per thread
+    // converter items of 4 values of a chunk: (row, half) for the first 128 rows, then the last 2R rows
+    static constexpr int MAIN = MROWS * 2 / 32;           // items per lane
+    static constexpr int EXTRA = 2 * R * 2;               // lanes with one more
+    static_assert(EXTRA <= 32, "items of a lane");
     // shared memory map
     static constexpr int OFF_STAGE = 1024;
-    static constexpr int OFF_OP = OFF_STAGE + STAGES * STAGE_BYTES;       // [2 bufs][hi,lo]
-    static constexpr int OFF_B = OFF_OP + 4 * OP_BYTES;                   // [K][hi,lo]
+    static constexpr int OFF_OP = OFF_STAGE + STAGES * STAGE_BYTES;       // [CGRP][hi,lo]
+    static constexpr int OFF_B = OFF_OP + CGRP * 2 * OP_BYTES;            // [K][hi,lo]
     static constexpr int SMEM = OFF_B + ((2 * K * B_BYTES + 1023) & ~1023);
 };
 
@@ -94,39 +106,34 @@ struct TcArgs {
 struct TcHeader {
     uint64_t stage_full[STAGES];
     uint64_t stage_empty[STAGES];
-    uint64_t op_full[2];
-    uint64_t op_empty[2];
+    uint64_t op_full[CGRP];
     uint64_t d_full[3];
     uint64_t d_free[3];
     uint64_t drain;
     uint32_t tmem_base;
     int abort_flag;
-    int conv_ok;
     int sc[SC_RING];     // per-plane scale exponents written by the converters
-    int dsc[3];          // scale exponent of the plane in each TMEM buffer
-    float red[2][4];     // converter max reduction
+    float red[CGRP][2][CONV_WARPS];   // converter max reduction; negative: the warp gave up
 };
 static_assert(sizeof(TcHeader) <= 1024, "header");
 
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo)
+// tcgen05 shared-memory matrix descriptor, no swizzle, K-major canonical layout of 8-row x 16-byte
+// core matrices.  Low word: start address and leading (K) byte offset, >> 4; high word: stride
+// (M/N) byte offset 128 >> 4 and the fixed value 0b001 in its bits 14-16, the same for every operand.
+constexpr uint32_t DESC_HI = (128 >> 4) | (1u << 14);
+__device__ __forceinline__ uint32_t umma_desc(uint32_t saddr, uint32_t lbo)
 {
-    // tcgen05 shared-memory matrix descriptor, no swizzle, K-major canonical layout of
-    // 8-row x 16-byte core matrices: start, leading (K) byte offset, stride (M/N) byte
-    // offset, all >> 4; bits 46-48 hold the fixed value 0b001.
-    uint64_t d = static_cast<uint64_t>((saddr >> 4) & 0x3FFF);
-    d |= static_cast<uint64_t>((lbo >> 4) & 0x3FFF) << 16;
-    d |= static_cast<uint64_t>((sbo >> 4) & 0x3FFF) << 32;
-    d |= static_cast<uint64_t>(1) << 46;
-    return d;
+    return ((saddr >> 4) & 0x3FFF) | (((lbo >> 4) & 0x3FFF) << 16);
 }
 
-__device__ __forceinline__ void umma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate)
+template <bool ACC>
+__device__ __forceinline__ void umma_f16(uint32_t dtmem, uint32_t adesc, uint32_t bdesc, uint32_t idesc)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "mov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(dtmem),
+        "r"(adesc), "r"(bdesc), "r"(idesc), "n"(ACC ? 1 : 0), "n"(DESC_HI)
         : "memory");
 }
 
@@ -137,24 +144,8 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar)
             smem_u32(bar))
         : "memory");
 }
-
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
-{
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 // 16 columns of this warp's 32 lanes into v[0..15]; complete after tmem_wait_ld()
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float* v)
@@ -202,7 +193,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     k_tc(const __grid_constant__ CUtensorMap tmap, const TcArgs p, const TcW<K> W)
 {
     using C = TcCfg<K>;
-    constexpr int R = C::R, ROWS = C::ROWS, N = C::N;
+    constexpr int R = C::R, N = C::N;
     extern __shared__ __align__(1024) unsigned char smem[];
     TcHeader& h = *reinterpret_cast<TcHeader*>(smem);
     volatile int* abort_flag = &h.abort_flag;
@@ -214,10 +205,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             mbar_init(&h.stage_full[s], 1);
             mbar_init(&h.stage_empty[s], 1);
         }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&h.op_full[b], 1);
-            mbar_init(&h.op_empty[b], 1);
-        }
+        for (int b = 0; b < CGRP; ++b) mbar_init(&h.op_full[b], CONV_WARPS);
         for (int b = 0; b < C::DBUF; ++b) {
             mbar_init(&h.d_full[b], 2);          // MMA completion + the issuer's scale hand-off
             mbar_init(&h.d_free[b], NEPI / 32);
@@ -236,8 +224,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
     {
         // T_b hi/lo, K-major [kc][n][8 halves] with n = (slot c, j) and entry kk = kc*8 + e.
-        // CAT: one matrix per b with 2N rows per kc chunk (rows [0,N) hi, [N,2N) lo);
-        // otherwise the hi matrix followed by the lo matrix.
+        // The hi matrix is followed by the lo matrix.
         const float sw = pow2f(p.wexp);
         __half* B = reinterpret_cast<__half*>(smem + C::OFF_B);
         const int per_b = 2 * N * 8;
@@ -250,14 +237,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             if (c < K && a >= 0 && a < K) v = W.w[(c * K + b) * K + a] * sw;
             const __half hi = __float2half_rn(v);
             const __half lo = __float2half_rn(v - __half2float(hi));
-            if (C::CAT) {
-                __half* Bb = B + b * 2 * (C::B_BYTES / 2);
-                Bb[(kc * 2 * N + n) * 8 + e] = hi;
-                Bb[(kc * 2 * N + N + n) * 8 + e] = lo;
-            } else {
-                B[(2 * b + 0) * (C::B_BYTES / 2) + rem] = hi;
-                B[(2 * b + 1) * (C::B_BYTES / 2) + rem] = lo;
-            }
+            B[(2 * b + 0) * (C::B_BYTES / 2) + rem] = hi;
+            B[(2 * b + 1) * (C::B_BYTES / 2) + rem] = lo;
         }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -267,199 +248,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const uint32_t tbase = h.tmem_base;
     const uint32_t sbase = smem_u32(smem);
 
-    if (warp == 0) {
-        // ---------------- TMA producer
-        if (lane == 0) {
-            uint32_t g = 0;
-            bool ok = true;
-            for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
-                const int xi = item % p.items_x, yi = (item / p.items_x) % p.items_y;
-                const int zv = item / (p.items_x * p.items_y);
-                const int vol = zv / p.items_z, zi = zv - vol * p.items_z;
-                const int x0 = xi * 8 * XT, y0 = yi * MROWS, zc0 = zi * p.zchunk;
-                const int zc1 = min(zc0 + p.zchunk, p.nz);
-                const int nplanes = zc1 - zc0 + 2 * R;
-                for (int it = 0; it < nplanes; ++it, ++g) {
-                    const int s = g % STAGES;
-                    if (g >= STAGES && !wait_or_abort(&h.stage_empty[s], ((g / STAGES) - 1) & 1,
-                                                      abort_flag, p.status)) {
-                        ok = false;
-                        break;
-                    }
-                    mbar_arrive_expect_tx(&h.stage_full[s], C::STAGE_TX);
-                    tma_load_4d(smem + C::OFF_STAGE + s * C::STAGE_BYTES, &tmap, &h.stage_full[s],
-                                x0 - 4, y0 - R, clampi(zc0 - R + it, 0, p.nz - 1), vol);
-                }
-            }
-            // drain: every issued load completes its stage (bounded, no abort check)
-            for (uint32_t q = (g > STAGES ? g - STAGES : 0); q < g; ++q)
-                mbar_wait(&h.stage_full[q % STAGES], (q / STAGES) & 1);
-        }
-    } else if (warp == 1) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
-            // idesc: D f32, A f16, B f16, both K-major, N >> 3 at bit 17, M >> 4 at bit 24
-            const uint32_t idesc = (1u << 4) | (static_cast<uint32_t>(N >> 3) << 17) |
-                                   (static_cast<uint32_t>(MROWS >> 4) << 24);
-            const uint32_t idesc2 = (1u << 4) | (static_cast<uint32_t>((2 * N) >> 3) << 17) |
-                                    (static_cast<uint32_t>(MROWS >> 4) << 24);
-            // Descriptors are built once: B per (dy, part) for the whole kernel, A as a per-
-            // buffer base to which each MMA adds its compile-time offset in the 14-bit start
-            // address field (addresses stay below 256 KB, so the add never carries out), so
-            // the issuing thread spends about one instruction per MMA.
-            uint64_t bdesc[2 * K];
-#pragma unroll
-            for (int b = 0; b < K; ++b) {
-                const uint32_t bb = sbase + C::OFF_B + 2 * b * C::B_BYTES;
-                if (C::CAT) {
-                    bdesc[2 * b] = umma_desc(bb, 2 * N * 16, 128);
-                    bdesc[2 * b + 1] = bdesc[2 * b];
-                } else {
-                    bdesc[2 * b] = umma_desc(bb, N * 16, 128);
-                    bdesc[2 * b + 1] = umma_desc(bb + C::B_BYTES, N * 16, 128);
-                }
-            }
-            uint64_t abase[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) abase[q] = umma_desc(sbase + C::OFF_OP + q * C::OP_BYTES, ROWS * 16, 128);
-            uint32_t g = 0;
-            bool ok = true;
-            for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
-                const int zi = item / (p.items_x * p.items_y) % p.items_z;
-                const int zc0 = zi * p.zchunk, zc1 = min(zc0 + p.zchunk, p.nz);
-                const int nplanes = zc1 - zc0 + 2 * R;
-                for (int it = 0; it < nplanes; ++it, ++g) {
-                    const int ob = g & 1, db = g % C::DBUF;
-                    if (!wait_or_abort(&h.op_full[ob], (g >> 1) & 1, abort_flag, p.status) ||
-                        (g >= C::DBUF && !wait_or_abort(&h.d_free[db], ((g / C::DBUF) - 1) & 1,
-                                                        abort_flag, p.status))) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint64_t ahi0 = ob ? abase[2] : abase[0];
-                    const uint64_t alo0 = ob ? abase[3] : abase[1];
-                    const uint32_t d0 = tbase + static_cast<uint32_t>(db * XT * C::DN);
-#pragma unroll
-                    for (int t = 0; t < XT; ++t) {
-                        const uint32_t dt = d0 + static_cast<uint32_t>(t * C::DN);
-#pragma unroll
-                        for (int b = 0; b < K; ++b) {
-                            const uint64_t aoff = static_cast<uint64_t>((t * (ROWS * 16) + b * 16) >> 4);
-                            if (C::CAT) {
-                                umma_f16(dt, ahi0 + aoff, bdesc[2 * b], idesc2, b > 0 ? 1u : 0u);
-                                umma_f16(dt, alo0 + aoff, bdesc[2 * b], idesc, 1u);
-                            } else {
-                                umma_f16(dt, ahi0 + aoff, bdesc[2 * b], idesc, b > 0 ? 1u : 0u);
-                                umma_f16(dt, ahi0 + aoff, bdesc[2 * b + 1], idesc, 1u);
-                                umma_f16(dt, alo0 + aoff, bdesc[2 * b], idesc, 1u);
-                            }
-                        }
-                    }
-                    umma_commit(&h.op_empty[ob]);
-                    h.dsc[db] = h.sc[g % SC_RING];
-                    umma_commit(&h.d_full[db]);
-                    mbar_arrive(&h.d_full[db]);
-                }
-            }
-            // drain: all MMAs issued so far complete before TMEM is released
-            umma_commit(&h.drain);
-            mbar_wait(&h.drain, 0);
-        }
-    } else if (warp < EPI_WARP0) {
-        // ---------------- converters: f32 tile -> fp16 hi/lo operand planes
-        const int ct = tid - CONV_WARP0 * 32;           // 0..127
-        const int cw = ct / 32;
-        uint32_t g = 0;
-        for (int item = blockIdx.x; item < p.nitems; item += gridDim.x) {
-            const int xi = item % p.items_x, yi = (item / p.items_x) % p.items_y;
-            const int zi = item / (p.items_x * p.items_y) % p.items_z;
-            const int x0 = xi * 8 * XT, y0 = yi * MROWS, zc0 = zi * p.zchunk;
-            const int zc1 = min(zc0 + p.zchunk, p.nz);
-            const int nplanes = zc1 - zc0 + 2 * R;
-            bool ok = true;
-            for (int it = 0; it < nplanes; ++it, ++g) {
-                const int s = g % STAGES, ob = g & 1;
-                if (ct == 0) {
-                    bool w = wait_or_abort(&h.stage_full[s], (g / STAGES) & 1, abort_flag, p.status);
-                    if (w && g >= 2)
-                        w = wait_or_abort(&h.op_empty[ob], ((g >> 1) - 1) & 1, abort_flag, p.status);
-                    h.conv_ok = w ? 1 : 0;
-                }
-                named_sync(1, NCONV);
-                if (!*reinterpret_cast<volatile int*>(&h.conv_ok)) {
-                    ok = false;
-                    break;
-                }
-                const float* st = reinterpret_cast<const float*>(smem + C::OFF_STAGE + s * C::STAGE_BYTES);
-                float v[C::UPT][4];
-                float mx = 0.f;
-#pragma unroll
-                for (int q = 0; q < C::UPT; ++q) {
-                    const int u = ct + q * NCONV;
-                    if (u < C::UNITS) {
-                        const int hf = u & 1, cr = u >> 1;
-                        const int ch = cr / ROWS, row = cr - ch * ROWS;
-                        const int gy = clampi(y0 - R + row, 0, p.ny - 1);
-                        const float* sr = st + (gy - (y0 - R)) * (NCH * 8);
-                        const int gx0 = x0 - 4 + 8 * ch + 4 * hf;
-                        if (gx0 >= 0 && gx0 + 3 < p.nx) {
-                            const float4 a = *reinterpret_cast<const float4*>(sr + 8 * ch + 4 * hf);
-                            v[q][0] = a.x; v[q][1] = a.y; v[q][2] = a.z; v[q][3] = a.w;
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                v[q][e] = sr[clampi(gx0 + e, 0, p.nx - 1) - (x0 - 4)];
-                        }
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fabsf(v[q][e]));
-                    }
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                if ((ct & 31) == 0) h.red[g & 1][cw] = mx;
-                named_sync(1, NCONV);
-                if (ct == 0) mbar_arrive(&h.stage_empty[s]);
-                mx = fmaxf(fmaxf(h.red[g & 1][0], h.red[g & 1][1]), fmaxf(h.red[g & 1][2], h.red[g & 1][3]));
-                // scale exponent: max|x| * 2^e in [2^13, 2^14)
-                int ex = 0;
-                int e = 0;
-                if (mx > 0.f && mx <= 3.0e38f) {
-                    frexpf(mx, &ex);
-                    e = min(max(14 - ex, -100), 100);
-                }
-                if (ct == 0) h.sc[g % SC_RING] = e;
-                const float sx = pow2f(e);
-                unsigned char* ohi = smem + C::OFF_OP + (2 * ob + 0) * C::OP_BYTES;
-                unsigned char* olo = smem + C::OFF_OP + (2 * ob + 1) * C::OP_BYTES;
-#pragma unroll
-                for (int q = 0; q < C::UPT; ++q) {
-                    const int u = ct + q * NCONV;
-                    if (u < C::UNITS) {
-                        uint32_t hw[2], lw[2];
-#pragma unroll
-                        for (int e2 = 0; e2 < 2; ++e2) {
-                            const float a = v[q][2 * e2] * sx, b = v[q][2 * e2 + 1] * sx;
-                            const __half ah = __float2half_rn(a), bh = __float2half_rn(b);
-                            const __half al = __float2half_rn(a - __half2float(ah));
-                            const __half bl = __float2half_rn(b - __half2float(bh));
-                            hw[e2] = static_cast<uint32_t>(__half_as_ushort(ah)) |
-                                     (static_cast<uint32_t>(__half_as_ushort(bh)) << 16);
-                            lw[e2] = static_cast<uint32_t>(__half_as_ushort(al)) |
-                                     (static_cast<uint32_t>(__half_as_ushort(bl)) << 16);
-                        }
-                        // item u = (chunk, row, half) lands at chunk*ROWS*16 + row*16 + half*8 = u*8
-                        *reinterpret_cast<uint2*>(ohi + u * 8) = make_uint2(hw[0], hw[1]);
-                        *reinterpret_cast<uint2*>(olo + u * 8) = make_uint2(lw[0], lw[1]);
-                    }
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                named_sync(1, NCONV);
-                if (ct == 0) mbar_arrive(&h.op_full[ob]);
-            }
-            if (!ok) break;
-        }
-    } else {
+    if (warp >= EPI_WARP0) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_EPI));
         // ---------------- epilogue
         const int et = tid - EPI_WARP0 * 32;            // 0..255
         const int t = et / 128;                          // x tile
@@ -467,7 +257,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int m = quad * 32 + lane;                  // output row within the tile
         const uint32_t lane_addr = static_cast<uint32_t>(quad * 32) << 16;
         uint32_t g = 0;
-        float acc[K][8];
+        float2 acc[K][4];
         bool ok = true;
         for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
             const int xi = item % p.items_x, yi = (item / p.items_x) % p.items_y;
@@ -482,7 +272,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll
             for (int c = 0; c < K; ++c)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[c][j] = 0.f;
+                for (int j = 0; j < 4; ++j) acc[c][j] = make_float2(0.f, 0.f);
 
             auto plane = [&](const int it, const int u) {
                 const int db = g % C::DBUF;
@@ -494,7 +284,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     return;
                 }
                 tc_fence_after();
-                const float inv = pow2f(-(h.dsc[db] + p.wexp));
+                const float inv = pow2f(-(h.sc[g % SC_RING] + p.wexp));
                 const uint32_t col = tbase + lane_addr + static_cast<uint32_t>((db * XT + t) * C::DN);
                 // two 16-column loads in flight per wait: slots 4q .. 4q+3
 #pragma unroll
@@ -510,7 +300,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                         if (c < K && (h2 < 2 || two)) {
                             const int sl = ((u - c + R) % K + K) % K;
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) acc[sl][j] = fmaf(d[8 * h2 + j], inv, acc[sl][j]);
+                            for (int j = 0; j < 4; ++j)
+                                acc[sl][j] = __ffma2_rn(make_float2(d[8 * h2 + 2 * j], d[8 * h2 + 2 * j + 1]),
+                                                        make_float2(inv, inv), acc[sl][j]);
                         }
                     }
                 }
@@ -522,16 +314,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     const int oz = zc0 + it - 2 * R;
                     float* d = dst + (static_cast<int64_t>(oz) * p.ny + oy) * p.nx + ox;
                     if (nvalid >= 8 && ((reinterpret_cast<uintptr_t>(d) & 15) == 0)) {
-                        reinterpret_cast<float4*>(d)[0] = make_float4(acc[sl0][0], acc[sl0][1], acc[sl0][2], acc[sl0][3]);
-                        reinterpret_cast<float4*>(d)[1] = make_float4(acc[sl0][4], acc[sl0][5], acc[sl0][6], acc[sl0][7]);
+                        reinterpret_cast<float4*>(d)[0] = make_float4(acc[sl0][0].x, acc[sl0][0].y, acc[sl0][1].x, acc[sl0][1].y);
+                        reinterpret_cast<float4*>(d)[1] = make_float4(acc[sl0][2].x, acc[sl0][2].y, acc[sl0][3].x, acc[sl0][3].y);
                     } else {
 #pragma unroll
                         for (int j = 0; j < 8; ++j)
-                            if (j < nvalid) d[j] = acc[sl0][j];
+                            if (j < nvalid) d[j] = j & 1 ? acc[sl0][j / 2].y : acc[sl0][j / 2].x;
                     }
                 }
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[sl0][j] = 0.f;
+                for (int j = 0; j < 4; ++j) acc[sl0][j] = make_float2(0.f, 0.f);
                 ++g;
             };
 
@@ -540,6 +332,209 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 for (int u = 0; u < K; ++u) {
                     if (g0 + u >= nplanes || !ok) break;
                     plane(g0 + u, u);
+                }
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_CONV));
+        if (warp == TMA_WARP) {
+            // ---------------- TMA producer
+            if (lane == 0) {
+                uint32_t g = 0;
+                bool ok = true;
+                for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
+                    const int xi = item % p.items_x, yi = (item / p.items_x) % p.items_y;
+                    const int zv = item / (p.items_x * p.items_y);
+                    const int vol = zv / p.items_z, zi = zv - vol * p.items_z;
+                    const int x0 = xi * 8 * XT, y0 = yi * MROWS, zc0 = zi * p.zchunk;
+                    const int zc1 = min(zc0 + p.zchunk, p.nz);
+                    const int nplanes = zc1 - zc0 + 2 * R;
+                    for (int it = 0; it < nplanes; ++it, ++g) {
+                        const int s = g % STAGES;
+                        if (g >= STAGES && !wait_or_abort(&h.stage_empty[s], ((g / STAGES) - 1) & 1,
+                                                          abort_flag, p.status)) {
+                            ok = false;
+                            break;
+                        }
+                        mbar_arrive_expect_tx(&h.stage_full[s], C::STAGE_TX);
+                        tma_load_4d(smem + C::OFF_STAGE + s * C::STAGE_BYTES, &tmap, &h.stage_full[s],
+                                    x0 - 4, y0 - R, clampi(zc0 - R + it, 0, p.nz - 1), vol);
+                    }
+                }
+                // drain: every issued load completes its stage (bounded, no abort check)
+                for (uint32_t q = (g > STAGES ? g - STAGES : 0); q < g; ++q)
+                    mbar_wait(&h.stage_full[q % STAGES], (q / STAGES) & 1);
+            }
+        } else if (warp == MMA_WARP) {
+            // ---------------- MMA issuer: lane 0 issues, the warp walks the planes together
+            {
+                // idesc: D f32, A f16, B f16, both K-major, N >> 3 at bit 17, M >> 4 at bit 24
+                constexpr uint32_t idesc = (1u << 4) | (static_cast<uint32_t>(N >> 3) << 17) |
+                                           (static_cast<uint32_t>(MROWS >> 4) << 24);
+                // Each MMA adds a compile-time offset to the start address field of two bases (addresses
+                // stay below 256 KB, so the add never carries out).
+                const uint32_t a0 = umma_desc(sbase + C::OFF_OP, C::CHUNK_BYTES);
+                const uint32_t b0 = umma_desc(sbase + C::OFF_B, N * 16);
+                const uint32_t tb = __shfl_sync(0xffffffffu, tbase, 0);
+                uint32_t g = 0;
+                bool ok = true;
+                for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
+                    const int zi = item / (p.items_x * p.items_y) % p.items_z;
+                    const int zc0 = zi * p.zchunk, zc1 = min(zc0 + p.zchunk, p.nz);
+                    const int nplanes = zc1 - zc0 + 2 * R;
+                    for (int it = 0; it < nplanes; ++it, ++g) {
+                        const uint32_t ob = g % CGRP, db = g % C::DBUF;
+                        int w = 1;
+                        if (lane == 0)
+                            w = wait_or_abort(&h.op_full[ob], (g / CGRP) & 1, abort_flag, p.status) &&
+                                (g < C::DBUF || wait_or_abort(&h.d_free[db], ((g / C::DBUF) - 1) & 1, abort_flag, p.status));
+                        if (!__shfl_sync(0xffffffffu, w, 0)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        if (lane == 0) {
+                            mbar_arrive(&h.d_full[db]);   // early: hands the plane's scale on to the epilogue
+                            const uint32_t ahi = a0 + ob * (2 * C::OP_BYTES >> 4), alo = ahi + (C::OP_BYTES >> 4);
+                            const uint32_t d0 = tb + db * (XT * C::DN);
+                            // (opaque, or the sums below are kept across planes and spilled)
+                            uint32_t b1 = b0;
+                            asm volatile("" : "+r"(b1));
+#pragma unroll
+                            for (int t = 0; t < XT; ++t) {
+#pragma unroll
+                                for (int b = 0; b < K; ++b) {
+                                    const uint32_t ao = (t * C::CHUNK_BYTES + b * 16) >> 4;
+                                    const uint32_t bh = b1 + (2 * b * C::B_BYTES >> 4), bl = bh + (C::B_BYTES >> 4);
+                                    if (b == 0)
+                                        umma_f16<false>(d0 + t * C::DN, ahi + ao, bh, idesc);
+                                    else
+                                        umma_f16<true>(d0 + t * C::DN, ahi + ao, bh, idesc);
+                                    umma_f16<true>(d0 + t * C::DN, ahi + ao, bl, idesc);
+                                    umma_f16<true>(d0 + t * C::DN, alo + ao, bh, idesc);
+                                }
+                            }
+                            umma_commit(&h.d_full[db]);   // also frees the operand buffer
+                        }
+                        __syncwarp();
+                    }
+                }
+                // drain: all MMAs issued so far complete before TMEM is released
+                if (lane == 0) {
+                    umma_commit(&h.drain);
+                    mbar_wait(&h.drain, 0);
+                }
+            }
+        } else if (warp < EPI_WARP0 && warp % 4 != MMA_WARP) {
+            // ---------------- converters: f32 tile -> fp16 hi/lo operand planes
+            // Group gr converts every third plane into operand buffer gr, while the MMAs read the others:
+            // the MMAs keep shared memory busy, so each step here takes a good part of a plane's time.
+            // Loading, scaling and splitting wait for the stage only.
+            const int gr = warp / 4;
+            const int cw = max(warp % 4 - 1, 0);            // the warp's chunk
+            const bool first = cw == 0 && lane == 0;        // of the group
+            // items: (row, half) with the half fastest, so that a quarter warp's 16-byte reads of the
+            // stage (rows 96 bytes apart) and its 8-byte writes of the operand planes touch distinct banks
+            const int half = lane & 1;
+            const bool extra = lane < C::EXTRA;             // one more: row 128 + lane / 2
+            unsigned char* const ohi = smem + C::OFF_OP + (2 * gr + 0) * C::OP_BYTES + cw * C::CHUNK_BYTES;
+            unsigned char* const olo = smem + C::OFF_OP + (2 * gr + 1) * C::OP_BYTES + cw * C::CHUNK_BYTES;
+            uint32_t g = 0;
+            bool ok = true, gone = false;
+            for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
+                const int xi = item % p.items_x, yi = (item / p.items_x) % p.items_y;
+                const int zi = item / (p.items_x * p.items_y) % p.items_z;
+                const int x0 = xi * 8 * XT, y0 = yi * MROWS, zc0 = zi * p.zchunk;
+                const int zc1 = min(zc0 + p.zchunk, p.nz);
+                const int nplanes = zc1 - zc0 + 2 * R;
+                // Rows are whole 16 bytes, so the lane's 4 columns are inside the volume together or
+                // outside it together; outside they repeat the first or the last column.
+                const int gx0 = x0 - 4 + 8 * cw + 4 * half;
+                const bool left = gx0 < 0, right = gx0 >= p.nx;
+                const int col = left ? 4 : right ? p.nx - x0 : 8 * cw + 4 * half;   // in the tile
+                const int ymax = p.ny - 1 - (y0 - R), ymin = R - y0;    // rows of the tile inside the volume
+                for (int it = 0; it < nplanes; ++it, ++g) {
+                    if (static_cast<int>(g % CGRP) != gr) continue;
+                    const int s = g % STAGES;
+                    int w = gone ? 0 : 1;
+                    if (lane == 0 && !gone)
+                        w = wait_or_abort(&h.stage_full[s], (g / STAGES) & 1, abort_flag, p.status) ? 1 : 0;
+                    w = __shfl_sync(0xffffffffu, w, 0);
+                    const float* st = reinterpret_cast<const float*>(smem + C::OFF_STAGE + s * C::STAGE_BYTES);
+                    float v[C::MAIN + 1][4];
+                    float mx = 0.f;
+                    auto fetch = [&](float (&o)[4], int row) {
+                        const float* sr = st + min(max(row, ymin), ymax) * (NCH * 8);
+                        const float4 a = *reinterpret_cast<const float4*>(sr + col);
+                        o[0] = right ? a.w : a.x;
+                        o[1] = left ? a.x : right ? a.w : a.y;
+                        o[2] = left ? a.x : right ? a.w : a.z;
+                        o[3] = left ? a.x : a.w;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) mx = fmaxf(mx, fabsf(o[e]));
+                    };
+                    if (w) {
+#pragma unroll
+                        for (int q = 0; q < C::MAIN; ++q) fetch(v[q], 16 * q + lane / 2);
+                        if (extra) fetch(v[C::MAIN], MROWS + lane / 2);
+                    }
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                    float* red = h.red[gr][(g / CGRP) & 1];
+                    if (lane == 0) red[cw] = w ? mx : -1.f;
+                    named_sync(1 + gr, NCONV);
+                    const float r0 = red[0], r1 = red[1], r2 = red[2];
+                    if (fminf(fminf(r0, r1), r2) < 0.f) {   // the group gives up together
+                        ok = false;
+                        break;
+                    }
+                    if (first) mbar_arrive(&h.stage_empty[s]);
+                    mx = fmaxf(fmaxf(r0, r1), r2);
+                    // scale exponent: max|x| * 2^e in [2^13, 2^14)
+                    int e = 0;
+                    if (mx > 0.f && mx <= 3.0e38f) e = min(max(140 - (__float_as_int(mx) >> 23), -100), 100);
+                    const float sx = pow2f(e);
+                    uint2 hi[C::MAIN + 1], lo[C::MAIN + 1];
+#pragma unroll
+                    for (int q = 0; q <= C::MAIN; ++q) {
+                        if (q == C::MAIN && !extra) continue;
+                        uint32_t hw[2], lw[2];
+#pragma unroll
+                        for (int e2 = 0; e2 < 2; ++e2) {
+                            const float2 a = __fmul2_rn(make_float2(v[q][2 * e2], v[q][2 * e2 + 1]), make_float2(sx, sx));
+                            const __half2 ah = __floats2half2_rn(a.x, a.y);
+                            const float2 af = __half22float2(ah);
+                            const float2 al = __ffma2_rn(af, make_float2(-1.f, -1.f), a);
+                            const __half2 ll = __floats2half2_rn(al.x, al.y);
+                            hw[e2] = *reinterpret_cast<const uint32_t*>(&ah);
+                            lw[e2] = *reinterpret_cast<const uint32_t*>(&ll);
+                        }
+                        hi[q] = make_uint2(hw[0], hw[1]);
+                        lo[q] = make_uint2(lw[0], lw[1]);
+                    }
+                    // the MMAs of the buffer's last plane are done (a warp that gives up here takes the
+                    // group out at its next plane)
+                    w = 1;
+                    if (g >= CGRP) {
+                        if (lane == 0)
+                            w = wait_or_abort(&h.d_full[(g - CGRP) % C::DBUF], ((g - CGRP) / C::DBUF) & 1, abort_flag,
+                                              p.status) ? 1 : 0;
+                        w = __shfl_sync(0xffffffffu, w, 0);
+                    }
+                    if (!w) {
+                        gone = true;
+                        continue;
+                    }
+#pragma unroll
+                    for (int q = 0; q <= C::MAIN; ++q) {
+                        if (q == C::MAIN && !extra) continue;
+                        *reinterpret_cast<uint2*>(ohi + q * 256 + lane * 8) = hi[q];
+                        *reinterpret_cast<uint2*>(olo + q * 256 + lane * 8) = lo[q];
+                    }
+                    if (first) h.sc[g % SC_RING] = e;
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&h.op_full[gr]);
                 }
             }
         }
@@ -595,6 +590,12 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx)
         return VKT_ERROR_UNSUPPORTED;
     cudaError_t e = cudaFuncSetAttribute(k_tc<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return from_cuda(e);
+    // the kernel's warpgroups hand registers on: it must have been built with as many as they count on
+    static const bool regs_ok = [] {
+        cudaFuncAttributes fa{};
+        return cudaFuncGetAttributes(&fa, k_tc<K>) == cudaSuccess && fa.numRegs >= REGS;
+    }();
+    if (!regs_ok) return VKT_ERROR_UNSUPPORTED;
     const int grid = static_cast<int>(std::min<long>(a.nitems, sms));
     if (ctx.debug & VKT_DEBUG_LOG)
         fprintf(stderr, "[vkt] tensor k=%d items=%d (%dx%dx%d, zchunk %d) grid=%d smem=%d\n", K,
