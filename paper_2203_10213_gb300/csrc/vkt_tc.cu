@@ -23,15 +23,16 @@
 //   warp 5         lane 0 issues TMA loads of f32 plane tiles
 //   warps 4g+0, 2, 3 (g < 3)   convert plane tiles to fp16 hi/lo operands (clamp-to-edge, scale)
 //   warps 12..19   epilogue: TMEM -> registers, z-march accumulate, store
-// What bounds it: an MMA of 128 x 64 x 16 reads 6 KB of shared memory, 48 of its 55 cycles, and a
-// plane of an item at k = 7 has 42 of them (2290 cycles of the 2980 it takes; the rest is the hand-off
-// between planes and the epilogue's and converters' share of shared memory).  Two things kept the
-// MMAs from that rate.  (1) Warps 1, 5, 9, ... share a scheduler: with converters among them an MMA took
-// 70 to 80 cycles to issue.  (2) A converter's loads and stores wait for shared memory behind the
-// MMAs, a plane takes a group 5800 cycles, so two operand buffers (and one group) ran dry; hence three
-// groups with a buffer each, and the registers moved from them to the epilogue (setmaxnreg).
-// 1024 x 1024 x 256, before and after: k = 5 1413 / 1087 us, k = 7 1655 / 1413, k = 9 2063 / 1752; 128^3, k = 7
-// 68 / 33.  No gain from: A operands on whole 128-byte lines, collector reuse of A, a second D.
+// What bounds it: an MMA of 128 x 64 x 16 reads 6 KB of shared memory, 48 of its 53 cycles, one of
+// 128 x 128 x 16 8 KB in 69; at k = 7 the 28 MMAs of an item's plane take 1710 of its 2420 cycles, the
+// rest is the hand-off between planes and the converters' share of shared memory.  What kept the MMAs
+// from that rate, with 1024 x 1024 x 256 at k = 5 / 7 / 9 1413 / 1655 / 2063 us and 128^3 at k = 7 68:
+// (1) Warps 1, 5, 9, ... share a scheduler: with converters among them an MMA took 70 to 80 cycles to
+// issue.  (2) A converter's loads and stores wait for shared memory behind the MMAs, a plane takes a
+// group 5800 cycles, so two operand buffers (and one group) ran dry; hence three groups with a buffer
+// each, and the registers moved from them to the epilogue (setmaxnreg).  Both: 1087 / 1413 / 1752, 33.
+// (3) STACK below: 967 / 1146, 28.5.
+// No gain from: A operands on whole 128-byte lines, collector reuse of A, issuing by the whole warp.
 // Every wait is bounded; on a timeout the CTA records it, drains what it issued and exits.
 #include <cuda_fp16.h>
 
@@ -66,8 +67,14 @@ struct TcCfg {
     static constexpr int ROWS = MROWS + 2 * R;            // input rows of a plane tile
     static constexpr int SLOTS = ((K + 1) / 2) * 2;       // even, so N is a multiple of 16
     static constexpr int N = SLOTS * 8;
-    static constexpr int DN = N;                         // TMEM columns per (buffer, x tile)
-    static constexpr int DBUF = 3;                       // TMEM accumulator buffers
+    // STACK: A_hi T_hi and A_hi T_lo are one MMA over the stacked operand [T_hi | T_lo] of 2N columns;
+    // D's columns [0, N) then hold the hi hi and lo hi products and [N, 2N) the hi lo ones.  An MMA's
+    // time is that of its shared memory reads below N = 128 (53 cycles at 64, 69 at 128), so a row
+    // offset takes 122 cycles instead of 160.  At k = 9 two buffers of 2N columns do not fit TMEM.
+    static constexpr bool STACK = K <= 7;
+    static constexpr int DN = STACK ? 2 * N : N;         // TMEM columns per (buffer, x tile)
+    static constexpr int DBUF = STACK ? 2 : 3;           // TMEM accumulator buffers
+    static_assert(STACK || DBUF == CGRP, "d_full stands in for op_empty");
     static_assert(DBUF * XT * DN <= 512, "TMEM holds 512 columns");
     static constexpr int TMEM_COLS = (DBUF * XT * DN <= 256) ? 256 : 512;
     static constexpr int STAGE_BYTES = ((ROWS * NCH * 8 * 4) + 1023) & ~1023;
@@ -107,6 +114,7 @@ struct TcHeader {
     uint64_t stage_full[STAGES];
     uint64_t stage_empty[STAGES];
     uint64_t op_full[CGRP];
+    uint64_t op_empty[CGRP];
     uint64_t d_full[3];
     uint64_t d_free[3];
     uint64_t drain;
@@ -205,7 +213,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             mbar_init(&h.stage_full[s], 1);
             mbar_init(&h.stage_empty[s], 1);
         }
-        for (int b = 0; b < CGRP; ++b) mbar_init(&h.op_full[b], CONV_WARPS);
+        for (int b = 0; b < CGRP; ++b) {
+            mbar_init(&h.op_full[b], CONV_WARPS);
+            mbar_init(&h.op_empty[b], 1);
+        }
         for (int b = 0; b < C::DBUF; ++b) {
             mbar_init(&h.d_full[b], 2);          // MMA completion + the issuer's scale hand-off
             mbar_init(&h.d_free[b], NEPI / 32);
@@ -224,7 +235,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
     {
         // T_b hi/lo, K-major [kc][n][8 halves] with n = (slot c, j) and entry kk = kc*8 + e.
-        // The hi matrix is followed by the lo matrix.
+        // STACK: 2N rows per kc chunk, the hi matrix's first; otherwise the hi matrix, then the lo matrix.
         const float sw = pow2f(p.wexp);
         __half* B = reinterpret_cast<__half*>(smem + C::OFF_B);
         const int per_b = 2 * N * 8;
@@ -237,8 +248,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             if (c < K && a >= 0 && a < K) v = W.w[(c * K + b) * K + a] * sw;
             const __half hi = __float2half_rn(v);
             const __half lo = __float2half_rn(v - __half2float(hi));
-            B[(2 * b + 0) * (C::B_BYTES / 2) + rem] = hi;
-            B[(2 * b + 1) * (C::B_BYTES / 2) + rem] = lo;
+            __half* Bb = B + 2 * b * (C::B_BYTES / 2);
+            if (C::STACK) {
+                Bb[(kc * 2 * N + n) * 8 + e] = hi;
+                Bb[(kc * 2 * N + N + n) * 8 + e] = lo;
+            } else {
+                Bb[rem] = hi;
+                Bb[C::B_BYTES / 2 + rem] = lo;
+            }
         }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -286,23 +303,27 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 tc_fence_after();
                 const float inv = pow2f(-(h.sc[g % SC_RING] + p.wexp));
                 const uint32_t col = tbase + lane_addr + static_cast<uint32_t>((db * XT + t) * C::DN);
-                // two 16-column loads in flight per wait: slots 4q .. 4q+3
+                // two 16-column loads in flight per wait: slots 4q .. 4q+3, or both parts of 2q and 2q+1
+                constexpr int SPL = C::STACK ? 2 : 4;
 #pragma unroll
-                for (int q = 0; q < (N / 16 + 1) / 2; ++q) {
+                for (int q = 0; q < (C::SLOTS + SPL - 1) / SPL; ++q) {
                     float d[32];
-                    const bool two = 2 * q + 1 < N / 16;
-                    tmem_ld16_nowait(col + 32 * q, d);
-                    if (two) tmem_ld16_nowait(col + 32 * q + 16, d + 16);
+                    const bool two = C::STACK || 2 * q + 1 < N / 16;
+                    tmem_ld16_nowait(col + 8 * SPL * q, d);
+                    if (two) tmem_ld16_nowait(col + 8 * SPL * q + (C::STACK ? N : 16), d + 16);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int h2 = 0; h2 < 4; ++h2) {
-                        const int c = 4 * q + h2;
+                    for (int h2 = 0; h2 < SPL; ++h2) {
+                        const int c = SPL * q + h2;
                         if (c < K && (h2 < 2 || two)) {
                             const int sl = ((u - c + R) % K + K) % K;
 #pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                acc[sl][j] = __ffma2_rn(make_float2(d[8 * h2 + 2 * j], d[8 * h2 + 2 * j + 1]),
-                                                        make_float2(inv, inv), acc[sl][j]);
+                            for (int j = 0; j < 4; ++j) {
+                                float2 v = make_float2(d[8 * h2 + 2 * j], d[8 * h2 + 2 * j + 1]);
+                                if (C::STACK)
+                                    v = __fadd2_rn(v, make_float2(d[16 + 8 * h2 + 2 * j], d[16 + 8 * h2 + 2 * j + 1]));
+                                acc[sl][j] = __ffma2_rn(v, make_float2(inv, inv), acc[sl][j]);
+                            }
                         }
                     }
                 }
@@ -369,12 +390,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             // ---------------- MMA issuer: lane 0 issues, the warp walks the planes together
             {
                 // idesc: D f32, A f16, B f16, both K-major, N >> 3 at bit 17, M >> 4 at bit 24
-                constexpr uint32_t idesc = (1u << 4) | (static_cast<uint32_t>(N >> 3) << 17) |
-                                           (static_cast<uint32_t>(MROWS >> 4) << 24);
+                auto idesc_of = [](int n) {
+                    return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(MROWS >> 4) << 24);
+                };
+                const uint32_t idesc = idesc_of(N), idesc2 = idesc_of(2 * N);
                 // Each MMA adds a compile-time offset to the start address field of two bases (addresses
                 // stay below 256 KB, so the add never carries out).
                 const uint32_t a0 = umma_desc(sbase + C::OFF_OP, C::CHUNK_BYTES);
-                const uint32_t b0 = umma_desc(sbase + C::OFF_B, N * 16);
+                const uint32_t b0 = umma_desc(sbase + C::OFF_B, (C::STACK ? 2 : 1) * N * 16);
                 const uint32_t tb = __shfl_sync(0xffffffffu, tbase, 0);
                 uint32_t g = 0;
                 bool ok = true;
@@ -406,15 +429,24 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                                 for (int b = 0; b < K; ++b) {
                                     const uint32_t ao = (t * C::CHUNK_BYTES + b * 16) >> 4;
                                     const uint32_t bh = b1 + (2 * b * C::B_BYTES >> 4), bl = bh + (C::B_BYTES >> 4);
-                                    if (b == 0)
-                                        umma_f16<false>(d0 + t * C::DN, ahi + ao, bh, idesc);
-                                    else
-                                        umma_f16<true>(d0 + t * C::DN, ahi + ao, bh, idesc);
-                                    umma_f16<true>(d0 + t * C::DN, ahi + ao, bl, idesc);
-                                    umma_f16<true>(d0 + t * C::DN, alo + ao, bh, idesc);
+                                    const uint32_t dt = d0 + t * C::DN;
+                                    if (C::STACK) {
+                                        if (b == 0)
+                                            umma_f16<false>(dt, ahi + ao, bh, idesc2);
+                                        else
+                                            umma_f16<true>(dt, ahi + ao, bh, idesc2);
+                                    } else {
+                                        if (b == 0)
+                                            umma_f16<false>(dt, ahi + ao, bh, idesc);
+                                        else
+                                            umma_f16<true>(dt, ahi + ao, bh, idesc);
+                                        umma_f16<true>(dt, ahi + ao, bl, idesc);
+                                    }
+                                    umma_f16<true>(dt, alo + ao, bh, idesc);
                                 }
                             }
-                            umma_commit(&h.d_full[db]);   // also frees the operand buffer
+                            if (C::STACK) umma_commit(&h.op_empty[ob]);
+                            umma_commit(&h.d_full[db]);
                         }
                         __syncwarp();
                     }
@@ -517,7 +549,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     w = 1;
                     if (g >= CGRP) {
                         if (lane == 0)
-                            w = wait_or_abort(&h.d_full[(g - CGRP) % C::DBUF], ((g - CGRP) / C::DBUF) & 1, abort_flag,
+                            // (three D buffers: plane g's barrier is the one that plane g - 3 completes next)
+                            w = wait_or_abort(C::STACK ? &h.op_empty[gr] : &h.d_full[gr], ((g / CGRP) - 1) & 1, abort_flag,
                                               p.status) ? 1 : 0;
                         w = __shfl_sync(0xffffffffu, w, 0);
                     }
