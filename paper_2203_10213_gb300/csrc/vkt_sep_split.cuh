@@ -21,7 +21,7 @@
 // thread per voxel, so the codes are the Dot2 codes bit for bit; about 1 in 10^4 voxels is.
 // (Evaluating the listed voxels where they occur would leave 31 lanes waiting each time.)
 // 8 FMAs per tap of the three passes instead of 32 flops: 94 instructions per voxel at k = 5
-// where Dot2 has 200.  512 x 512 x 256 uint16 -> uint16, k = 5: 635 -> 311 us (0.86 TB/s); bound
+// where Dot2 has 200.  512 x 512 x 256 uint16 -> uint16, k = 5: 635 -> 298 us (0.90 TB/s); bound
 // by latency at 16 warps per SM (issue 47 %, barrier and fixed-latency stalls), of which the
 // listed voxels take 17 us (45 us with a thread per voxel also for short lists).
 #pragma once

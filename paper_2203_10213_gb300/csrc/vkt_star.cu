@@ -9,7 +9,7 @@
 // 128 columns x 4 rows, a CTA 128 x 32, marching through z; a stage is refilled once every warp
 // has arrived at its "empty" barrier.
 // The taps are added in the order of the general kernel, (z-1) (y-1) (x-1) (0) (x+1) (y+1) (z+1), so the
-// float32 sums are the same.  Bound by HBM traffic: 512^3 uint8 -> float32 194 -> 111 us (6.0 TB/s of
+// float32 sums are the same.  Bound by HBM traffic: 512^3 uint8 -> float32 194 -> 108 us (6.2 TB/s of
 // the 6.8 a copy reaches), into uint8 codes 1637 (Dot2) -> 181 us.
 #include <algorithm>
 #include <cstdio>
