@@ -413,7 +413,7 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
             const int oy = y0 + ty * RY + i;
             if (it >= 2 * R && oy < yend && nvalid > 0) {
                 const int64_t idx = (static_cast<int64_t>(pfirst + it - R) * J.ny + oy) * J.nx + ox;
-                store_row<RX>(J.dst, dfmt, idx, nvalid, rowv, J.a0, J.a1, J.qmax, first, nwide);
+                store_row<RX, (K < 9)>(J.dst, dfmt, idx, nvalid, rowv, J.a0, J.a1, J.qmax, first, nwide);
             }
         };
         if constexpr (PAIR) {
