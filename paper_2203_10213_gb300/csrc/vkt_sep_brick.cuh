@@ -46,6 +46,7 @@ struct Job {
     int zchunk;
     int use_tma;
     int rows;          // no tensor map: stages filled by row copies (issue_rows)
+    int withhold_first;    // fault injection (split brick): the first plane's load is never issued
     // output region: bricks start at (ox0, oy0, oz0) and store the voxels with x in
     // [sx0, sx1), y < sy1, z < sz1 (the whole volume: set_whole_volume)
     int ox0, oy0, oz0;

@@ -21,7 +21,7 @@
 // thread per voxel, so the codes are the Dot2 codes bit for bit; about 1 in 10^4 voxels is.
 // (Evaluating the listed voxels where they occur would leave 31 lanes waiting each time.)
 // 8 FMAs per tap of the three passes instead of 32 flops: 94 instructions per voxel at k = 5
-// where Dot2 has 200.  512 x 512 x 256 uint16 -> uint16, k = 5: 635 -> 298 us (0.90 TB/s); bound
+// where Dot2 has 200.  512 x 512 x 256 uint16 -> uint16, k = 5: 635 -> 304 us (0.88 TB/s); bound
 // by latency at 16 warps per SM (issue 47 %, barrier and fixed-latency stalls), of which the
 // listed voxels take 17 us (45 us with a thread per voxel also for short lists).
 #pragma once
@@ -235,6 +235,7 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
     const uint64_t vol_bytes = static_cast<uint64_t>(J.nx) * J.ny * J.nz * ES;
     if (tma && tid == 0) {
         for (int s = 0; s < STAGES && s < nplanes; ++s, ++issued) {
+            if (s == 0 && J.withhold_first) continue;
             const uint32_t q = g0 + s;
             mbar_arrive_expect_tx(&bars[q % STAGES], txb);
             tma_load_3d(raw + (q % STAGES) * rawb, tmap, &bars[q % STAGES], x0 - XA, y0 - R,
@@ -250,7 +251,6 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
         if (tid == 0)
             for (int s = 0; s < STAGES && s < nplanes; ++s, ++issued) mbar_arrive(&bars[(g0 + s) % STAGES]);
     }
-    int pend = -1;   // a stage refilled by row copies, to be given its arrival
 
     // (H, L) of the K output planes in progress; slot K-1-c takes tap c, slot 0 completes
     float2 aH[K][RX / 2], aL[K][RX / 2];
@@ -265,7 +265,13 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
     const int first = (ROI && J.sx0 > ox) ? J.sx0 - ox : 0;   // leading columns outside the region
     const int yend = ROI ? J.sy1 : J.ny;
     const bool xin = x0 - R >= 0 && x0 + TX - 1 + R <= J.nx - 1;
-    bool failed = false;
+    // A wait ends by the clock, so one warp may give up a wait that another one sees end.  All lanes
+    // of a warp give up together (GONE), and a warp that is gone makes no more arrivals, so no other
+    // one gets past the wait for the plane it did not reach: they are gone one limit later at the
+    // latest.  Until then it takes part in the CTA's barriers only, of which the votes end the
+    // brick for all warps at once (FAILED): one every SPLIT_CHECK planes and one after the last.
+    enum { RUNS, GONE, FAILED };
+    int state = RUNS;
 
     // evaluates the listed voxels again (all threads; the caller synchronises around it): a
     // thread per voxel if there are many, a warp per voxel if few
@@ -288,22 +294,24 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
         }
     };
 
-    // The x pass of plane `it` into tile it % 3.
+    // waits for the source plane `it`
+    auto loaded = [&](const int it) {
+        return !(tma || rows) || mbar_wait(&bars[(g0 + it) % STAGES], ((g0 + it) / STAGES) & 1);
+    };
+
+    // The x pass of plane `it` (which is loaded) into tile it % 3.
     auto x_pass = [&](const int it) {
         const uint32_t q = g0 + it;
         const int s = q % STAGES;
         const unsigned char* rs = raw + s * rawb;
-        bool ok = true;
-        if (tma || rows) {
-            ok = mbar_wait(&bars[s], (q / STAGES) & 1);
-        } else {
+        if (!tma && !rows) {
             fill_raw_plain<Geo, NT>(const_cast<unsigned char*>(rs), J.src, SF, J.nx, J.ny, J.nz, x0,
                                     y0, pfirst + it, tid);
             __syncthreads();
         }
         float* Th = T + (it % 3) * 2 * FH * TX;
         float* Tl = Th + FH * TX;
-        if (ok) {
+        {
             const uint32_t zterm = static_cast<uint32_t>(clampi(pfirst + it, 0, J.nz - 1)) *
                                    static_cast<uint32_t>(J.ny) * static_cast<uint32_t>(J.nx);
 #pragma unroll
@@ -339,7 +347,6 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
         }
         __syncwarp();
         if ((tid & 31) == 0) mbar_arrive(xbar);
-        return ok;
     };
 
     // Plane `it`: the x pass of the plane after it, then its own y and z passes.  A warp arrives at
@@ -351,16 +358,15 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
     auto plane = [&](const int it, const int u) {
         const uint32_t q = g0 + it;
         const int s = q % STAGES;
-        if (!mbar_wait(xbar, (gx + it) & 1)) {
-            failed = true;
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait(xbar, (gx + it) & 1) && (it + 1 >= nplanes || loaded(it + 1)))) {
+            state = GONE;
             return;
         }
         // stage s is read
-        if (rows && tid == 0 && pend >= 0) {
-            mbar_arrive(&bars[pend]);
+        if (rows && tid == 0 && it > 0 && it - 1 + STAGES < nplanes) {
+            mbar_arrive(&bars[(q - 1) % STAGES]);   // of the refill before this one
             ++issued;
         }
-        pend = -1;
         if (tma && tid == 0 && it + STAGES < nplanes) {
             mbar_arrive_expect_tx(&bars[s], txb);
             tma_load_3d(raw + s * rawb, tmap, &bars[s], x0 - XA, y0 - R,
@@ -370,18 +376,18 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
             // all threads; the arrival follows the next plane's wait
             copy_rows<Geo, BULK, SF>(raw + s * rawb, &bars[s], J.src, vol_bytes, SF, J.nx, J.ny, J.nz, x0,
                                 y0, pfirst + it + STAGES, tid);
-            pend = s;
         }
         if (it % SPLIT_CHECK == SPLIT_CHECK - 1 && __syncthreads_or(*count >= SPLIT_LIST)) {
+            if (__syncthreads_or(0)) {   // a warp is gone
+                state = FAILED;
+                return;
+            }
             work_off();
             __syncthreads();
             if (tid == 0) *count = 0;
             __syncthreads();
         }
-        if (it + 1 < nplanes && !x_pass(it + 1)) {
-            failed = true;
-            return;
-        }
+        if (it + 1 < nplanes) x_pass(it + 1);
         const float* Th = T + (it % 3) * 2 * FH * TX;
         const float* Tl = Th + FH * TX;
         // y pass
@@ -458,41 +464,64 @@ __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUt
                 }
         }
     };
-    failed = !x_pass(0);
-    if constexpr (ROTZ) {
+    int at = 0;   // the plane a warp is at, or was when it left (-1: before the first)
+    if (__all_sync(0xFFFFFFFFu, loaded(0))) {
+        x_pass(0);
+        if constexpr (ROTZ) {
 #pragma unroll 1
-        for (int it = 0; it < nplanes && !failed; ++it) plane(it, 0);
-    } else {
-#pragma unroll 1
-        for (int g = 0; g < nplanes && !failed; g += K) {
-#pragma unroll
-            for (int u = 0; u < K; ++u) {
-                if (g + u >= nplanes || failed) break;
-                plane(g + u, u);
+            for (; at < nplanes; ++at) {
+                plane(at, 0);
+                if (state != RUNS) break;
             }
+        } else {
+#pragma unroll 1
+            for (; at < nplanes && state == RUNS; at += K) {
+#pragma unroll
+                for (int u = 0; u < K; ++u) {
+                    if (at + u >= nplanes) break;
+                    plane(at + u, u);
+                    if (state != RUNS) {
+                        at += u - K;
+                        break;
+                    }
+                }
+            }
+        }
+    } else {
+        state = GONE;
+        at = -1;
+    }
+    // a warp that is gone: the barriers of the planes it does not take, up to a vote
+#pragma unroll 1
+    for (int it = max(at, 0); state == GONE && it < nplanes; ++it) {
+        if (it % SPLIT_CHECK == SPLIT_CHECK - 1) {
+            __syncthreads_or(1);
+            __syncthreads_or(1);
+            state = FAILED;
+        } else if (!tma && !rows && it + 1 < nplanes) {
+            __syncthreads();
         }
     }
     if (tma || rows) gplane = g0 + nplanes;
     xphase = gx + nplanes;
     if (!tma) fence_proxy_async();   // a next brick's tensor-map loads may refill these stages
-    // (all threads wait for the same stages and for one another, so they fail together, within the
-    // limit of a wait)
-    if (failed) {
-        __syncthreads();
+    // the last vote; also, every voxel is listed and its first code stored
+    if (state != FAILED && __syncthreads_or(state == GONE)) state = FAILED;
+    if (state == FAILED) {
         if (tid == 0) {
             atomicOr(status, STATUS_TIMEOUT);
-            // a refill whose copies are in flight still needs its arrival before the drain
-            if (pend >= 0) {
-                mbar_arrive(&bars[pend]);
-                ++issued;
-            }
+            // the refills after the planes before `at` and, by other warps that got past their wait
+            // for it, after `at`: those whose copies are in flight still need their arrival before
+            // the drain
+            for (; rows && issued < min(at + STAGES + 1, nplanes); ++issued)
+                mbar_arrive(&bars[(g0 + issued) % STAGES]);
             for (int it = issued - 1; it >= 0 && it >= issued - STAGES; --it)
-                mbar_wait(&bars[(g0 + it) % STAGES], ((g0 + it) / STAGES) & 1);
+                if (it != 0 || !J.withhold_first)
+                    mbar_wait(&bars[(g0 + it) % STAGES], ((g0 + it) / STAGES) & 1);
         }
         __syncthreads();
         return false;
     }
-    __syncthreads();   // every voxel is listed (and its first code stored)
     work_off();
     __syncthreads();   // before a next brick clears the list
     return true;

@@ -191,7 +191,7 @@ vktError launch_k(const Job& job, const float* gx, const float* gy, const float*
     // Integer codes that need more than FP32: the split evaluation where it suits the job, else
     // Dot2.  k >= 3 (at k = 1 Dot2 is three products), integer sources (a float32 voxel has no unit
     // that the weights' parts could be exact in), and a filter that make_split_plan accepts.
-    // 512 x 512 x 256 uint16, k = 5: 635 us by Dot2, 298 us by the split.
+    // 512 x 512 x 256 uint16, k = 5: 635 us by Dot2, 304 us by the split.
     sep::SplitW<K> S;
     bool use_split = false;
     auto split = &k_separable_split<(K < 3 ? 3 : K), FMT_U16, sep::LM_ANY, true>;
@@ -202,6 +202,7 @@ vktError launch_k(const Job& job, const float* gx, const float* gy, const float*
         else if (!job.roi) split = J.use_tma ? k_separable_split<K, FMT_U16, sep::LM_TMA>
                                              : k_separable_split<K, FMT_U16, sep::LM_ANY>;
         if (use_split) smem = sep::smem_bytes_split<K>(job.sfmt, J.rows != 0);
+        J.withhold_first = use_split && (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) ? 1 : 0;
     }
     // z chunks sized for whole waves of the CTAs the chosen kernel keeps resident
     int per_sm = 1;
