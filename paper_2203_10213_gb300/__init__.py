@@ -102,33 +102,58 @@ def set_policy(stream=None, path=None, debug=None, print_times=None) -> None:
 
 
 class policy(contextlib.ContextDecorator):
-    """Temporarily sets the calling thread's execution policy (None: keep the setting).  The
-    policy is set, and put back, only where it differs from the thread's (a call on the thread's
-    own stream makes one library call here instead of four)."""
+    """Temporarily sets the calling thread's execution policy (None: keep the setting).  The policy
+    found on entry is put back on exit, whatever the block did to it; it is set, and put back, only
+    where it differs from the thread's."""
 
     def __init__(self, stream=None, path=None, debug=None, print_times=None):
         self._args = stream, path, debug, print_times
+        self._found = []     # the policy at each entry that is still open
 
     def _recreate_cm(self):
         return policy(*self._args)
 
-    def __enter__(self):
+    def _enter(self):
+        """Sets the policy; returns the one found and whether it differed."""
         stream, path, debug, print_times = self._args
         old = get_policy()
         new = (_stream_handle(stream),
                old.path if path is None else PATHS[path] if isinstance(path, str) else int(path),
                old.debug if debug is None else int(debug),
                old.printTimes if print_times is None else int(bool(print_times)))
-        self._old = None
-        if new != (old.stream or 0, old.path, old.debug, old.printTimes):
+        differs = new != _fields(old)
+        if differs:
             check(_lib.vktSetThreadExecutionPolicy(
                 ExecutionPolicy(new[0], new[3], new[2], new[1])))
-            self._old = old
+        return old, differs
+
+    def __enter__(self):
+        self._found.append(self._enter()[0])
 
     def __exit__(self, *exc):
-        if self._old is not None:
-            check(_lib.vktSetThreadExecutionPolicy(self._old))
+        old = self._found.pop()
+        if _fields(get_policy()) != _fields(old):
+            check(_lib.vktSetThreadExecutionPolicy(old))
         return False
+
+
+class _call_policy(policy):
+    """The policy around one library call: nothing in the block changes it, so one that did not
+    differ on entry need not be looked at again (a call on the thread's own stream makes one
+    library call here instead of four)."""
+
+    def __enter__(self):
+        self._found.append(self._enter())
+
+    def __exit__(self, *exc):
+        old, differs = self._found.pop()
+        if differs:
+            check(_lib.vktSetThreadExecutionPolicy(old))
+        return False
+
+
+def _fields(p) -> tuple:
+    return p.stream or 0, p.path, p.debug, p.printTimes
 
 
 def _stream_handle(stream) -> int:
@@ -372,7 +397,7 @@ def apply_filter(dst: StructuredVolume, src: StructuredVolume, filt: Filter, pat
     """Enqueues dst = filter(src) on `stream` (default: torch's current stream); path None
     keeps the thread policy's path.  roi ((x0, y0, z0), (x1, y1, z1)): only the voxels of
     that half-open box are written (vktApplyFilterRangeSV)."""
-    with policy(stream=stream, path=path):
+    with _call_policy(stream=stream, path=path):
         if roi is None:
             check(_lib.vktApplyFilterSV(dst.handle, src.handle, filt.handle), "vktApplyFilterSV")
         else:
@@ -390,7 +415,7 @@ def apply_filter_batch(dsts, srcs, filters, stream=None) -> None:
     d = arr(*(v.handle.value for v in dsts))
     s = arr(*(v.handle.value for v in srcs))
     f = arr(*(x.handle.value for x in filters))
-    with policy(stream=stream):
+    with _call_policy(stream=stream):
         check(_lib.vktApplyFilterBatchSV(n, d, s, f), "vktApplyFilterBatchSV")
 
 
@@ -399,7 +424,7 @@ def apply_filter_backward(grad_src, grad_weights, grad_dst: StructuredVolume,
     """grad_src: StructuredVolume or None; grad_weights: float32 CUDA tensor (k^3) or None."""
     gs = grad_src.handle if grad_src is not None else None
     gw = ctypes.c_void_p(grad_weights.data_ptr()) if grad_weights is not None else None
-    with policy(stream=stream):
+    with _call_policy(stream=stream):
         check(_lib.vktApplyFilterBackwardSV(gs, gw, grad_dst.handle, src.handle, filt.handle),
               "vktApplyFilterBackwardSV")
 
@@ -416,7 +441,7 @@ def apply_filter_backward_batch(grad_srcs, grad_weights, grad_dsts, srcs, filt: 
     gd = arr(*(v.handle.value for v in grad_dsts))
     sv = arr(*(v.handle.value for v in srcs))
     gw = ctypes.c_void_p(grad_weights.data_ptr()) if grad_weights is not None else None
-    with policy(stream=stream):
+    with _call_policy(stream=stream):
         check(_lib.vktApplyFilterBackwardBatchSV(n, gs, gw, gd, sv, filt.handle),
               "vktApplyFilterBackwardBatchSV")
 
@@ -449,7 +474,7 @@ def brick_decompose(src_t, brick, ghost: int = 0, src_range=(0.0, 1.0), stream=N
                 pointers.append(t.data_ptr())
                 dims += (int(dx), int(dy), int(dz))
     with _Views(pointers, dims, _fmt_of_dtype(src_t.dtype), *src_range, keep=tensors) as views:
-        with policy(stream=stream):
+        with _call_policy(stream=stream):
             check(_lib.vktBrickDecomposeSV(views, len(tensors), src.handle, bx, by, bz, int(ghost)),
                   "vktBrickDecomposeSV")
     return tensors
@@ -481,7 +506,7 @@ def render(src_t, width: int, height: int, eye, center, up, fovy: float, step: f
     prm.background[:] = [float(x) for x in background]
     prm.lutSize = table.shape[0]
     prm.lut = table.ctypes.data_as(ctypes.POINTER(ctypes.c_float))
-    with policy(stream=stream):
+    with _call_policy(stream=stream):
         check(_lib.vktRenderSV(ctypes.c_void_p(out.data_ptr()), int(width), int(height), vol.handle,
                                ctypes.cast(ctypes.pointer(prm), ctypes.c_void_p)), "vktRenderSV")
     return out
@@ -495,7 +520,7 @@ def clahe3d(src_t, bricks, clip_limit: float, out=None, stream=None):
         out = torch.empty_like(src_t)
     src = StructuredVolume.from_tensor(src_t)
     dst = StructuredVolume.from_tensor(out)
-    with policy(stream=stream):
+    with _call_policy(stream=stream):
         check(_lib.vktClahe3DSV(dst.handle, src.handle, *map(int, bricks), float(clip_limit)),
               "vktClahe3DSV")
     return out
@@ -536,7 +561,7 @@ def _autograd_function():
             filt = Filter.dense(w_host)
             y = torch.empty_like(xb)
             n = xb.shape[0]
-            with _Views.of_batch(xb) as vx, _Views.of_batch(y) as vy, policy(path=path):
+            with _Views.of_batch(xb) as vx, _Views.of_batch(y) as vy, _call_policy(path=path):
                 check(_lib.vktApplyFilterBatchSV(n, vy, vx, (ctypes.c_void_p * n)(*[filt.handle.value] * n)),
                       "vktApplyFilterBatchSV")
             ctx.save_for_backward(xb)
@@ -556,7 +581,7 @@ def _autograd_function():
                 k3 *= d
             gw = torch.empty(k3, dtype=torch.float32, device=xb.device) if need_w else None
             n = xb.shape[0]
-            with _Views.of_batch(xb) as vx, _Views.of_batch(gyb) as vgy, policy():
+            with _Views.of_batch(xb) as vx, _Views.of_batch(gyb) as vgy, _call_policy():
                 args = (ctypes.c_void_p(gw.data_ptr()) if need_w else None, vgy, vx, ctx.filt.handle)
                 if need_x:
                     with _Views.of_batch(gx) as vgx:
