@@ -92,9 +92,10 @@ struct Cell {
     float2 v[4];                     // rows (y, z) (y + 1, z) (y, z + 1) (y + 1, z + 1)
 };
 
-// x's cell along one axis: i with w = x - i in [0, 1], by rounding x - 1/2 to an integer in the
-// low bits of 1.5 * 2^23 + x - 1/2.  (At a whole x this may be the cell below with w = 1, whose
-// blend is the same voxel.)  BIG: axes of more than 2^21 voxels, where that has too few bits.
+// x's cell along one axis, the integer i at or below x, and w = x - i: x is rounded down to an integer
+// in the low bits of 1.5 * 2^23 + x.  (At a whole x the blend has to take that voxel with weight 1 and
+// the one above it with 0: 0 times an infinite voxel is NaN, so the cell below would not do.)
+// BIG: axes of more than 2^21 voxels, where that has too few bits.
 template <bool BIG>
 __device__ __forceinline__ int cell(float x, float& w)
 {
@@ -103,7 +104,7 @@ __device__ __forceinline__ int cell(float x, float& w)
         w = x - f;
         return static_cast<int>(f);
     }
-    const float s = (x - 0.5f) + 12582912.f;
+    const float s = __fadd_rd(x, 12582912.f);
     w = x - (s - 12582912.f);
     return static_cast<int>(__float_as_uint(s)) - 0x4B400000;
 }
@@ -182,7 +183,7 @@ template <int FMT, typename Off, bool REUSE>
 __global__ void __launch_bounds__(BX* BY) k_render(const __grid_constant__ RenderArgs a, float* __restrict__ rgba)
 {
     // entry i and its difference to the next (GENERAL: the next itself, which may be infinite); the
-    // last entry's next is itself, since fi = n - 1 may round to cell n - 1 with w = 0
+    // last entry's next is itself, since fi = n - 1 lies in cell n - 1 with w = 0
     constexpr bool GENERAL = sizeof(Off) == 8;
     __shared__ float4 lut[VKT_RENDER_MAX_LUT][2];
     const int tid = threadIdx.y * BX + threadIdx.x;
@@ -238,7 +239,11 @@ __global__ void __launch_bounds__(BX* BY) k_render(const __grid_constant__ Rende
             const float un = sample_u<FMT, Off, REUSE>(a, ex + t * d[0], ey + t * d[1], ez + t * d[2], near);
             float w;
             const float fi = un * m;       // in [0, m], so its cell is in [0, m]
-            const int i0 = cell<false>(fi, w);
+            int i0 = cell<false>(fi, w);
+            if constexpr (GENERAL) {       // the last entry is the upper end of the cell before it
+                i0 = min(i0, a.lut_n - 2);
+                w = fi - static_cast<float>(i0);
+            }
             const float4 e = lut[i0][0], n = lut[i0][1];
             float cr, cg, cb, ca;
             if constexpr (GENERAL) {
