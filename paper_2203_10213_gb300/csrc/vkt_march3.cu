@@ -32,10 +32,11 @@ constexpr int SMEM = 128 + STAGES * STAGE;
 struct MarchArgs {
     void* dst;
     int nx, ny, nz;
-    int dfmt, zchunk, gzv;      // gzv: z chunks per volume
+    int zchunk, gzv;            // gzv: z chunks per volume
     int64_t vs_dst;             // voxels from one volume's destination to the next
     float w[27];
     float a0, a1, qmax;
+    int withhold_first;         // fault injection: the first plane's load is never issued
     unsigned* status;
 };
 
@@ -67,9 +68,10 @@ __global__ void __launch_bounds__(NT, 4)
     int issued = 0;
     auto issue = [&](int it) {
         const int s = it % STAGES;
+        ++issued;
+        if (it == 0 && p.withhold_first) return;
         mbar_arrive_expect_tx(&full[s], Geo::raw_tx(FMT_F32));
         tma_load_4d(raw + s * STAGE, &tmap, &full[s], x0 - XA, y0 - R, clampi(pfirst + it, 0, p.nz - 1), vol);
-        ++issued;
     };
     if (tid == 0)
         for (int it = 0; it < STAGES && it < nplanes; ++it) issue(it);
@@ -163,21 +165,21 @@ __global__ void __launch_bounds__(NT, 4)
     if (!ok) atomicOr(p.status, STATUS_TIMEOUT);
     // every load issued is waited for before the CTA's shared memory is released
     if (tid == 0)
-        for (int it = std::max(0, issued - STAGES); it < issued; ++it) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
+        for (int it = std::max(0, issued - STAGES); it < issued; ++it)
+            if (it != 0 || !p.withhold_first) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
     __syncthreads();
 }
 
 }  // namespace
 
 // Launches the march where it serves the job: *taken false otherwise.  Whole float32 volumes (a batch
-// of them evenly spaced) that a tensor map describes, into float32, wider than 32 columns and large
-// enough that 128 x 16 tiles in chunks of 8 planes give every SM its four CTAs; smaller ones have the
-// one-row shape of the general kernel.
+// of them evenly spaced) that a tensor map describes, into float32, at least one tile (128 columns)
+// wide with three quarters of the tiles' columns in use, and large enough that 128 x 16 tiles in chunks
+// of 8 planes give every SM its four CTAs; smaller ones have the one-row shape of the general kernel.
 vktError launch_march3(const Job& job, const float* w, const Ctx& ctx, bool* taken)
 {
     *taken = false;
     if (job.roi || job.sfmt != FMT_F32 || job.dfmt != FMT_F32 || job.nx < TX) return VKT_NO_ERROR;
-    if (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) return VKT_NO_ERROR;   // the general kernel injects it
     const int nvol = std::max(job.nvol, 1);
     const int tx = (job.nx + TX - 1) / TX, ty = (job.ny + TY - 1) / TY;
     if (4 * static_cast<long>(job.nx) < 3L * tx * TX) return VKT_NO_ERROR;
@@ -191,12 +193,12 @@ vktError launch_march3(const Job& job, const float* w, const Ctx& ctx, bool* tak
     a.nx = job.nx;
     a.ny = job.ny;
     a.nz = job.nz;
-    a.dfmt = job.dfmt;
     a.vs_dst = job.vs_dst;
     for (int i = 0; i < 27; ++i) a.w[i] = w[i];
     a.a0 = job.a0;
     a.a1 = job.a1;
     a.qmax = job.qmax;
+    a.withhold_first = (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) ? 1 : 0;
     a.status = ctx.status;
     int per_sm = 1;
     const vktError ve = prepare_kernel(ctx, reinterpret_cast<const void*>(k_march3), NT, SMEM, &per_sm);

@@ -36,6 +36,7 @@ struct StarArgs {
     float zm, ym, xm, c, xp, yp, zp;   // the taps
     float a0, a1, qmax;
     float whole, frac;                 // exact codes: whole + frac + sum
+    int withhold_first;                // fault injection: the first plane's load is never issued
     unsigned* status;
 };
 
@@ -76,9 +77,10 @@ __global__ void __launch_bounds__(NT, 2)
     int issued = 0;
     auto issue = [&](int it) {
         const int s = it % STAGES;
+        ++issued;
+        if (it == 0 && p.withhold_first) return;
         mbar_arrive_expect_tx(&full[s], G::PITCH * G::ROWS);
         tma_load_3d(raw + s * G::STAGE, &tmap, &full[s], x0 - G::XA, y0 - 1, clampi(zc0 - 1 + it, 0, p.nz - 1));
-        ++issued;
     };
     if (tid == 0)
         for (int it = 0; it < STAGES && it < nplanes; ++it) issue(it);
@@ -202,19 +204,19 @@ __global__ void __launch_bounds__(NT, 2)
     // every load issued is waited for before the CTA's shared memory is released (those of a
     // finished march have been read)
     if (tid == 0)
-        for (int it = std::max(0, issued - STAGES); it < issued; ++it) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
+        for (int it = std::max(0, issued - STAGES); it < issued; ++it)
+            if (it != 0 || !p.withhold_first) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
     __syncthreads();
 }
 
 }  // namespace
 
-// Whether the job is a 3^3 filter with taps on the axes only, over one whole integer volume that
-// a tensor map describes, into an aligned destination whose codes FP32 or exact sums decide; *exact
-// then says which.
+// Whether the job is a 3^3 filter with taps on the axes only, over one whole integer volume into an
+// aligned destination whose codes FP32 decides, or exact sums with the weights of `plan` (job.comp).
+// launch_star then asks for a tensor map of the volume.
 static bool star_job(const Job& job, const float* w, const Ctx& ctx, ListPlan& plan)
 {
     if (job.roi || job.nvol > 1 || job.sfmt == FMT_F32) return false;
-    if (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) return false;   // the general kernel injects it
     for (int c = 0; c < 3; ++c)
         for (int b = 0; b < 3; ++b)
             for (int a = 0; a < 3; ++a)
@@ -257,6 +259,7 @@ vktError launch_star(const Job& job, const float* w, const Ctx& ctx, bool* taken
     a.qmax = job.qmax;
     a.whole = job.comp ? plan.whole : 0.f;
     a.frac = job.comp ? plan.frac : 0.f;
+    a.withhold_first = (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) ? 1 : 0;
     a.status = ctx.status;
     const int out = job.dfmt == FMT_F32 ? OUT_F32 : job.comp ? OUT_EXACT_CODE : OUT_FP32_CODE;
     auto kern = u8 ? (out == OUT_F32 ? k_star<FMT_U8, OUT_F32>

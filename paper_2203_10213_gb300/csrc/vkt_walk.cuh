@@ -40,6 +40,7 @@ struct Args {
     int nx, ny, nz;
     int dfmt, zchunk;
     float a0, a1, qmax;
+    int withhold_first;    // fault injection: the first plane's load is never issued
     unsigned* status;
 };
 
@@ -83,9 +84,10 @@ __global__ void __launch_bounds__(NT, 3)
     int issued = 0;
     auto issue = [&](int it) {
         const int s = it % STAGES;
+        ++issued;
+        if (it == 0 && p.withhold_first) return;
         mbar_arrive_expect_tx(&full[s], Geo::raw_tx(SF));
         tma_load_3d(raw + s * C::STAGE, &tmap, &full[s], x0 - XA, y0 - R, clampi(pfirst + it, 0, p.nz - 1));
-        ++issued;
     };
     if (tid == 0)
         for (int it = 0; it < STAGES && it < nplanes; ++it) issue(it);
@@ -229,7 +231,8 @@ __global__ void __launch_bounds__(NT, 3)
     if (!ok) atomicOr(p.status, STATUS_TIMEOUT);
     // every load issued is waited for before the CTA's shared memory is released
     if (tid == 0)
-        for (int it = std::max(0, issued - STAGES); it < issued; ++it) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
+        for (int it = std::max(0, issued - STAGES); it < issued; ++it)
+            if (it != 0 || !p.withhold_first) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
     __syncthreads();
 }
 
@@ -286,6 +289,7 @@ vktError launch_walk_k(const Job& job, const float* gx, const float* gy, const f
     a.a0 = job.a0;
     a.a1 = job.a1;
     a.qmax = job.qmax;
+    a.withhold_first = (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) ? 1 : 0;
     a.status = ctx.status;
     W<K> G;
     for (int i = 0; i < K; ++i) {

@@ -14,7 +14,11 @@ pytestmark = pytest.mark.gpu
 if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
 
-GAUSS5 = vkt.Filter.gaussian(5, 1.5)
+GAUSS3, GAUSS5 = vkt.Filter.gaussian(3, 1.0), vkt.Filter.gaussian(5, 1.5)
+CROSS = np.zeros((3, 3, 3), np.float32)
+CROSS[1, 1, :] = CROSS[1, :, 1] = CROSS[:, 1, 1] = 0.125
+STAR = vkt.Filter.dense(CROSS)
+DENSE3 = vkt.Filter.dense(np.random.RandomState(1).standard_normal((3, 3, 3)).astype(np.float32))
 
 # what the log calls the kernel, (nz, ny, nx), source, destination, filter, path.  The split brick takes
 # three planes (no vote of its warps before the last plane) and many.
@@ -22,6 +26,12 @@ CASES = [
     ("separable-split", (3, 33, 136), torch.uint16, torch.uint16, GAUSS5, "separable"),
     ("separable-split", (70, 33, 136), torch.uint16, torch.uint16, GAUSS5, "separable"),
     ("separable-split", (20, 18, 64), torch.uint8, torch.uint16, GAUSS5, "separable"),
+    ("direct-star", (24, 32, 48), torch.uint8, torch.float32, STAR, "direct"),
+    ("direct-star", (3, 33, 136), torch.uint16, torch.float32, STAR, "direct"),
+    ("direct-march", (64, 1216, 128), torch.float32, torch.float32, DENSE3, "direct"),
+    ("separable-walk", (64, 1216, 128), torch.uint8, torch.float32, GAUSS3, "separable"),
+    ("separable-walk", (1, 33, 136), torch.float32, torch.float32, GAUSS3, "separable"),
+    ("separable-walk", (30, 17, 64), torch.float32, torch.float32, GAUSS5, "separable"),
 ]
 
 
