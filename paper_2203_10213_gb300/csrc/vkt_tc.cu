@@ -583,6 +583,21 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
 }
 
+// The kernel's warpgroups hand registers on: it must have been built with as many as they count on.
+// Where it was not, tensor_available says so and a call that may choose takes the direct path.
+// (Without a device there is no answer, and no launch either.)
+template <int K>
+bool registers_fit()
+{
+    static const bool fit = [] {
+        cudaFuncAttributes fa{};
+        if (cudaFuncGetAttributes(&fa, k_tc<K>) == cudaSuccess) return fa.numRegs >= REGS;
+        cudaGetLastError();
+        return true;
+    }();
+    return fit;
+}
+
 template <int K>
 vktError launch_k(const Job& job, const float* w, const Ctx& ctx)
 {
@@ -623,12 +638,7 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx)
         return VKT_ERROR_UNSUPPORTED;
     cudaError_t e = cudaFuncSetAttribute(k_tc<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return from_cuda(e);
-    // the kernel's warpgroups hand registers on: it must have been built with as many as they count on
-    static const bool regs_ok = [] {
-        cudaFuncAttributes fa{};
-        return cudaFuncGetAttributes(&fa, k_tc<K>) == cudaSuccess && fa.numRegs >= REGS;
-    }();
-    if (!regs_ok) return VKT_ERROR_UNSUPPORTED;
+    if (!registers_fit<K>()) return VKT_ERROR_UNSUPPORTED;
     const int grid = static_cast<int>(std::min<long>(a.nitems, sms));
     if (ctx.debug & VKT_DEBUG_LOG)
         fprintf(stderr, "[vkt] tensor k=%d items=%d (%dx%dx%d, zchunk %d) grid=%d smem=%d\n", K,
@@ -648,6 +658,8 @@ vktError tensor_available(const vktStructuredVolume_impl* dst, const vktStructur
     if (f->k != 5 && f->k != 7 && f->k != 9) return VKT_ERROR_UNSUPPORTED;
     if (src->dims[0] % 4 != 0 || reinterpret_cast<uintptr_t>(src->data) % 16 != 0)
         return VKT_ERROR_UNSUPPORTED;   // rows must be describable by a TMA tensor map
+    if (!(f->k == 5 ? registers_fit<5>() : f->k == 7 ? registers_fit<7>() : registers_fit<9>()))
+        return VKT_ERROR_UNSUPPORTED;
     return VKT_NO_ERROR;
 }
 
