@@ -443,7 +443,8 @@ extern "C" vktError vktClahe3DSV(vktStructuredVolume dst, vktStructuredVolume sr
         fprintf(stderr, "[vkt] clahe3d %dx%dx%d bricks %dx%dx%d (%dx%dx%d voxels) limit=%lld blend=%s\n",
                 g.nx, g.ny, g.nz, bricksX, bricksY, bricksZ, g.sx, g.sy, g.sz,
                 static_cast<long long>(limit), by_cells ? "cells" : "voxels");
-    if (ctx.debug & VKT_DEBUG_LOG) fprintf(stderr, "[vkt] clahe3d histogram loads of %d bytes\n", vec);
+    if (ctx.debug & VKT_DEBUG_LOG)
+        fprintf(stderr, "[vkt] clahe3d histogram loads of %d bytes, %d CTAs per brick\n", vec, parts);
     const cudaError_t e1 = cudaFreeAsync(luts, ctx.stream);
     if (e == cudaSuccess) e = e1;
     return from_cuda(e);
