@@ -786,6 +786,34 @@ static std::string tune_key(const vktStructuredVolume_impl* dst, const vktStruct
     return buf;
 }
 
+// Whether n float32 volumes of these dims, filtered by a dense k = 5 filter that the tensor path can
+// evaluate in one launch, are done sooner by the direct path.  Either time is the planes that the
+// busiest SM marches through times what a plane takes there: on the tensor path (16 x 128 columns, one
+// CTA per SM) 1.03 us, and 8.5 us for the launch, the first plane and the last; on the direct path
+// (64 x 32 columns) 1.86, 3.03 or 4.05 us with one, two or three CTAs on that SM.  Measured over 174
+// cases of 1 to 8 volumes of 32^3 to 1024x1024x256, powers of two and not, these are within 10 % of
+// the times, and the path chosen is never the slower one by more than 2 %.  us, direct / tensor:
+// 64^3 9.3 / 20.6, four of them
+// 24.8 / 20.7; eight of 160x32x128 48.8 / 92.7 (a quarter of each tensor tile in use), of 132x100x96
+// 112 / 60, of 128^3 93 / 81; one 160x150x128 48 / 33 and eight 182 / 192; 512^3 620 / 499.
+// (At k = 7 the tensor path is the faster one throughout: two of 32^3 30.7 / 24.8.)
+static bool direct5_faster(const int32_t* dims, long n)
+{
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int nx = dims[0], ny = dims[1], nz = dims[2];
+    auto over = [](long a, long b) { return (a + b - 1) / b; };
+    const long columns = over(nx, 16) * over(ny, 128) * n;
+    const long tz = zchunk_waves(columns, nz, sms, 2);
+    const double tensor = 8.5 + 1.03 * static_cast<double>(over(columns * over(nz, tz), sms) * (tz + 4));
+    const long tiles = over(nx, 64) * over(ny, 32) * n;
+    const long dz = zchunk_direct(tiles, nz, sms, 3, 2);
+    const long ctas = tiles * over(nz, dz);
+    const double plane = ctas <= sms ? 1.86 : 2 * ctas <= 3L * sms ? 3.03 : 4.05;
+    return plane * static_cast<double>(over(ctas, 3L * sms) * (dz + 4)) < tensor;
+}
+
 // ApplyFilter on the whole volume (box == nullptr) or on the region
 // [box[0], box[3]) x [box[1], box[4]) x [box[2], box[5]) (validated by the caller).
 //
@@ -812,7 +840,7 @@ static vktError apply_filter(vktStructuredVolume dst, vktStructuredVolume src, v
     if (auto_path) {
         if (filter->separable)
             path = VKT_PATH_SEPARABLE;
-        else if (tensor_ok)
+        else if (tensor_ok && !(k == 5 && direct5_faster(src->dims, 1)))
             path = VKT_PATH_TENSOR;
         else
             path = VKT_PATH_DIRECT;
@@ -897,8 +925,8 @@ static vktError apply_filter(vktStructuredVolume dst, vktStructuredVolume src, v
                 cand[n].path = cpath;
                 cand[n++].zchunk = zs[i];
             }
-            if (path == VKT_PATH_TENSOR) {   // the other path at its rule's z chunks
-                cand[n].path = cpath;
+            if (path != VKT_PATH_SEPARABLE && tensor_ok) {   // the other path at its rule's z chunks
+                cand[n].path = path == VKT_PATH_TENSOR ? cpath : VKT_PATH_TENSOR;
                 cand[n++].zchunk = 0;
             }
             err = autotune_time(cand, n, [&](const TuneChoice& t) { return launch(t.path, t.zchunk); },
@@ -960,12 +988,11 @@ vktError vkt::apply_filter_multi(int32_t n, vktStructuredVolume* dst, vktStructu
         if (f->separable) return VKT_NO_ERROR;   // the persistent separable batch
         path = (f->k >= 5 && tensor_available(dst[0], src[0], f) == VKT_NO_ERROR) ? VKT_PATH_TENSOR
                                                                                   : VKT_PATH_DIRECT;
-        // at k = 5 the direct launch, whose smaller tiles fill the GPU better, is the faster one
-        // for volumes of a power of two (8 x 128^3: direct 92 us, tensor 124; 2 x 64^3: 20 and
-        // 28) and near it otherwise (4 x 132x100x96: 60 and 51); at k = 7 the tensor launch is
-        // (8 x 128^3: 326 and 137 us)
-        int64_t s = 0;
-        if (f->k == 5 && evenly_spaced(n, src, &s) && evenly_spaced(n, dst, &s)) path = VKT_PATH_DIRECT;
+        // one launch over all n volumes either way, so the tensor map has to describe their spacing
+        int64_t s = 0, d = 0;
+        if (path == VKT_PATH_TENSOR && f->k == 5 && evenly_spaced(n, src, &s) && evenly_spaced(n, dst, &d) &&
+            (s % 4 != 0 || direct5_faster(src[0]->dims, n)))
+            path = VKT_PATH_DIRECT;
     }
     if (path == VKT_PATH_SEPARABLE) return VKT_NO_ERROR;
     if (path == VKT_PATH_TENSOR) {
