@@ -85,11 +85,11 @@ typedef struct vktFilter_impl* vktFilter;
  * Fault injection for tests of failure detection: every CTA of the direct path, and of the
  * separable path of vktApplyFilterSV and its range form where it walks in registers (k = 3 and
  * 5) or evaluates integer codes from integer sources in split form, withholds the TMA load of
- * its first input plane, so its bounded wait for that plane runs out (after 2 s).  The CTA then
- * records the timeout in the device status word, waits for the loads it did issue and exits
- * without writing; the next vktSynchronize returns VKT_ERROR_DEVICE_TIMEOUT and the context
- * stays usable.  No other path reads this flag, and calls whose source cannot use a tensor map
- * (rows not 16-byte aligned) ignore it.
+ * its first input plane, or an arrival that its barrier counts on, so its bounded wait for that
+ * plane runs out (after 2 s).  The CTA then records the timeout in the device status word,
+ * waits for the loads it did issue and exits without writing; the next vktSynchronize returns
+ * VKT_ERROR_DEVICE_TIMEOUT and the context stays usable.  No other path reads this flag, and
+ * calls whose source cannot use a tensor map (rows not 16-byte aligned) ignore it.
  */
 #define VKT_DEBUG_INJECT_WAIT_TIMEOUT 2
 

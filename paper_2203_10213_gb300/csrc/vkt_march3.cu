@@ -33,10 +33,10 @@ struct MarchArgs {
     void* dst;
     int nx, ny, nz;
     int zchunk, gzv;            // gzv: z chunks per volume
+    int withhold;               // fault injection: arrivals that the first plane's wait lacks
     int64_t vs_dst;             // voxels from one volume's destination to the next
     float w[27];
     float a0, a1, qmax;
-    int withhold_first;         // fault injection: the first plane's load is never issued
     unsigned* status;
 };
 
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(NT, 4)
     float* dst = static_cast<float*>(p.dst) + vol * p.vs_dst;
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1);
+            mbar_init(&full[s], s == 0 ? 1 + p.withhold : 1);
             mbar_init(&empty[s], NT / 32);
         }
         fence_mbar_init();
@@ -68,10 +68,9 @@ __global__ void __launch_bounds__(NT, 4)
     int issued = 0;
     auto issue = [&](int it) {
         const int s = it % STAGES;
-        ++issued;
-        if (it == 0 && p.withhold_first) return;
         mbar_arrive_expect_tx(&full[s], Geo::raw_tx(FMT_F32));
         tma_load_4d(raw + s * STAGE, &tmap, &full[s], x0 - XA, y0 - R, clampi(pfirst + it, 0, p.nz - 1), vol);
+        ++issued;
     };
     if (tid == 0)
         for (int it = 0; it < STAGES && it < nplanes; ++it) issue(it);
@@ -163,11 +162,12 @@ __global__ void __launch_bounds__(NT, 4)
         if (!ok) break;
     }
     if (!ok) atomicOr(p.status, STATUS_TIMEOUT);
+    __syncthreads();   // every warp's march has ended
     // every load issued is waited for before the CTA's shared memory is released
-    if (tid == 0)
-        for (int it = std::max(0, issued - STAGES); it < issued; ++it)
-            if (it != 0 || !p.withhold_first) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
-    __syncthreads();
+    if (tid == 0) {
+        if (p.withhold) mbar_arrive(&full[0]);
+        for (int it = std::max(0, issued - STAGES); it < issued; ++it) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
+    }
 }
 
 }  // namespace
@@ -198,7 +198,7 @@ vktError launch_march3(const Job& job, const float* w, const Ctx& ctx, bool* tak
     a.a0 = job.a0;
     a.a1 = job.a1;
     a.qmax = job.qmax;
-    a.withhold_first = (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) ? 1 : 0;
+    a.withhold = (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) ? 1 : 0;
     a.status = ctx.status;
     int per_sm = 1;
     const vktError ve = prepare_kernel(ctx, reinterpret_cast<const void*>(k_march3), NT, SMEM, &per_sm);

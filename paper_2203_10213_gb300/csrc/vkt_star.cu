@@ -32,11 +32,12 @@ enum : int { OUT_F32 = 0, OUT_FP32_CODE = 1, OUT_EXACT_CODE = 2 };
 struct StarArgs {
     void* dst;
     int nx, ny, nz;
-    int dfmt, zchunk;
+    int zchunk;
+    int withhold;                      // fault injection: arrivals that the first plane's wait lacks
+    int dfmt;
     float zm, ym, xm, c, xp, yp, zp;   // the taps
     float a0, a1, qmax;
     float whole, frac;                 // exact codes: whole + frac + sum
-    int withhold_first;                // fault injection: the first plane's load is never issued
     unsigned* status;
 };
 
@@ -65,7 +66,7 @@ __global__ void __launch_bounds__(NT, 2)
     const int nplanes = zc1 - zc0 + 2;
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1);
+            mbar_init(&full[s], s == 0 ? 1 + p.withhold : 1);
             mbar_init(&empty[s], NT / 32);
         }
         fence_mbar_init();
@@ -77,10 +78,9 @@ __global__ void __launch_bounds__(NT, 2)
     int issued = 0;
     auto issue = [&](int it) {
         const int s = it % STAGES;
-        ++issued;
-        if (it == 0 && p.withhold_first) return;
         mbar_arrive_expect_tx(&full[s], G::PITCH * G::ROWS);
         tma_load_3d(raw + s * G::STAGE, &tmap, &full[s], x0 - G::XA, y0 - 1, clampi(zc0 - 1 + it, 0, p.nz - 1));
+        ++issued;
     };
     if (tid == 0)
         for (int it = 0; it < STAGES && it < nplanes; ++it) issue(it);
@@ -201,12 +201,12 @@ __global__ void __launch_bounds__(NT, 2)
         __syncwarp();
     }
     if (!ok) atomicOr(p.status, STATUS_TIMEOUT);
-    // every load issued is waited for before the CTA's shared memory is released (those of a
-    // finished march have been read)
-    if (tid == 0)
-        for (int it = std::max(0, issued - STAGES); it < issued; ++it)
-            if (it != 0 || !p.withhold_first) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
-    __syncthreads();
+    __syncthreads();   // every warp's march has ended
+    // every load issued is waited for before the CTA's shared memory is released
+    if (tid == 0) {
+        if (p.withhold) mbar_arrive(&full[0]);
+        for (int it = std::max(0, issued - STAGES); it < issued; ++it) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
+    }
 }
 
 }  // namespace
@@ -259,7 +259,7 @@ vktError launch_star(const Job& job, const float* w, const Ctx& ctx, bool* taken
     a.qmax = job.qmax;
     a.whole = job.comp ? plan.whole : 0.f;
     a.frac = job.comp ? plan.frac : 0.f;
-    a.withhold_first = (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) ? 1 : 0;
+    a.withhold = (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) ? 1 : 0;
     a.status = ctx.status;
     const int out = job.dfmt == FMT_F32 ? OUT_F32 : job.comp ? OUT_EXACT_CODE : OUT_FP32_CODE;
     auto kern = u8 ? (out == OUT_F32 ? k_star<FMT_U8, OUT_F32>

@@ -38,9 +38,10 @@ struct W {
 struct Args {
     void* dst;
     int nx, ny, nz;
-    int dfmt, zchunk;
+    int zchunk;
+    int withhold;          // fault injection: arrivals that the first plane's wait lacks
+    int dfmt;
     float a0, a1, qmax;
-    int withhold_first;    // fault injection: the first plane's load is never issued
     unsigned* status;
 };
 
@@ -72,7 +73,7 @@ __global__ void __launch_bounds__(NT, 3)
     const int nplanes = zc1 - zc0 + 2 * R, pfirst = zc0 - R;
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1);
+            mbar_init(&full[s], s == 0 ? 1 + p.withhold : 1);
             mbar_init(&empty[s], NT / 32);
         }
         fence_mbar_init();
@@ -84,10 +85,9 @@ __global__ void __launch_bounds__(NT, 3)
     int issued = 0;
     auto issue = [&](int it) {
         const int s = it % STAGES;
-        ++issued;
-        if (it == 0 && p.withhold_first) return;
         mbar_arrive_expect_tx(&full[s], Geo::raw_tx(SF));
         tma_load_3d(raw + s * C::STAGE, &tmap, &full[s], x0 - XA, y0 - R, clampi(pfirst + it, 0, p.nz - 1));
+        ++issued;
     };
     if (tid == 0)
         for (int it = 0; it < STAGES && it < nplanes; ++it) issue(it);
@@ -229,11 +229,12 @@ __global__ void __launch_bounds__(NT, 3)
         u = u + 1 == K ? 0 : u + 1;
     }
     if (!ok) atomicOr(p.status, STATUS_TIMEOUT);
+    __syncthreads();   // every warp's march has ended
     // every load issued is waited for before the CTA's shared memory is released
-    if (tid == 0)
-        for (int it = std::max(0, issued - STAGES); it < issued; ++it)
-            if (it != 0 || !p.withhold_first) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
-    __syncthreads();
+    if (tid == 0) {
+        if (p.withhold) mbar_arrive(&full[0]);
+        for (int it = std::max(0, issued - STAGES); it < issued; ++it) mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
+    }
 }
 
 }  // namespace walk
@@ -289,7 +290,7 @@ vktError launch_walk_k(const Job& job, const float* gx, const float* gy, const f
     a.a0 = job.a0;
     a.a1 = job.a1;
     a.qmax = job.qmax;
-    a.withhold_first = (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) ? 1 : 0;
+    a.withhold = (ctx.debug & VKT_DEBUG_INJECT_WAIT_TIMEOUT) ? 1 : 0;
     a.status = ctx.status;
     W<K> G;
     for (int i = 0; i < K; ++i) {
