@@ -113,22 +113,16 @@ class policy(contextlib.ContextDecorator):
     def _recreate_cm(self):
         return policy(*self._args)
 
-    def _enter(self):
-        """Sets the policy; returns the one found and whether it differed."""
+    def __enter__(self):
         stream, path, debug, print_times = self._args
         old = get_policy()
-        new = (_stream_handle(stream),
-               old.path if path is None else PATHS[path] if isinstance(path, str) else int(path),
+        new = (_stream_handle(stream), old.path if path is None else _path_number(path),
                old.debug if debug is None else int(debug),
                old.printTimes if print_times is None else int(bool(print_times)))
-        differs = new != _fields(old)
-        if differs:
+        if new != _fields(old):
             check(_lib.vktSetThreadExecutionPolicy(
                 ExecutionPolicy(new[0], new[3], new[2], new[1])))
-        return old, differs
-
-    def __enter__(self):
-        self._found.append(self._enter()[0])
+        self._found.append(old)
 
     def __exit__(self, *exc):
         old = self._found.pop()
@@ -137,19 +131,31 @@ class policy(contextlib.ContextDecorator):
         return False
 
 
-class _call_policy(policy):
+class _call_policy:
     """The policy around one library call: nothing in the block changes it, so one that did not
     differ on entry need not be looked at again (a call on the thread's own stream makes one
     library call here instead of four)."""
 
+    def __init__(self, stream=None, path=None):
+        self._stream, self._path = stream, path
+
     def __enter__(self):
-        self._found.append(self._enter())
+        self._old = None
+        old, path = get_policy(), self._path
+        stream = _stream_handle(self._stream)
+        path = old.path if path is None else _path_number(path)
+        if path != old.path or stream != (old.stream or 0):
+            check(_lib.vktSetThreadExecutionPolicy(ExecutionPolicy(stream, old.printTimes, old.debug, path)))
+            self._old = old
 
     def __exit__(self, *exc):
-        old, differs = self._found.pop()
-        if differs:
-            check(_lib.vktSetThreadExecutionPolicy(old))
+        if self._old is not None:
+            check(_lib.vktSetThreadExecutionPolicy(self._old))
         return False
+
+
+def _path_number(path) -> int:
+    return PATHS[path] if isinstance(path, str) else int(path)
 
 
 def _fields(p) -> tuple:
