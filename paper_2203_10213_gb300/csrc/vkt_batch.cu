@@ -382,8 +382,8 @@ vktError build_plan(Plan& P, int32_t n, vktStructuredVolume* dst, vktStructuredV
                                          raw_width(tx, J.sfmt), ty + 2 * ((J.k - 1) / 2), 1)
                         ? 1
                         : 0;
-        // rows that no tensor map can describe are still fetched asynchronously, as 16-byte
-        // blocks, when the volume starts on a 16-byte boundary
+        // rows that no tensor map can describe are still fetched asynchronously, one bulk copy
+        // per row (issue_rows_bulk), when the volume starts on a 16-byte boundary
         J.rows = (!J.use_tma && reinterpret_cast<uintptr_t>(J.src) % 16 == 0) ? 1 : 0;
         order.push_back({-static_cast<long>(J.k) * (J.zchunk + J.k - 1), static_cast<int>(j)});
     }

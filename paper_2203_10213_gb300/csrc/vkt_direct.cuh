@@ -131,11 +131,9 @@ __host__ __device__ constexpr size_t direct_smem_bytes(int sfmt, bool rows)
                            : 0);
 }
 
-// SF/DF: source and destination formats fixed at compile time (-1: read from the arguments);
-// LM: how stages are filled, fixed at compile time where known (the plane loop is unrolled,
-// so code for unused ways of loading costs instruction cache): 0 = from the arguments
-// (tensor map, row copies or plain loads), 1 = tensor map, 2 = row copies
+// how stages are filled: read from the arguments, by tensor map, by row copies
 constexpr int LM_ANY = 0, LM_TMA = 1, LM_ROWS = 2;
+
 // the Dot2 code of voxel (x, y, z): the taps in the order and with the operations of the
 // compensated kernel.  The voxels of a plane are loaded before its chain of K^2 steps, which
 // hides all but one load latency per plane.
@@ -178,6 +176,9 @@ __device__ __noinline__ unsigned dot2_voxel(const void* src, int sfmt, int nx, i
     return comp_code(s, e, a0, a0lo, a1, a1lo, qmax);
 }
 
+// SF/DF: source and destination formats fixed at compile time (-1: read from the arguments);
+// LM: how stages are filled, fixed at compile time where known (the plane loop is unrolled,
+// so code for unused ways of loading costs instruction cache).
 // ROI: the forward stores are bounded by the arguments' region fields; otherwise by the
 // volume (known at compile time to start at column 0).  MODE: see above; other than M_PLAIN
 // into an integer destination (forward only).

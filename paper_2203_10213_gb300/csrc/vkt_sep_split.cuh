@@ -134,8 +134,6 @@ __device__ __forceinline__ void regrid(float2& H, float2& L, float m)
     H = h;
 }
 
-// ROTZ: as in brick(); the accumulator slots are shifted after each plane, or the plane loop
-// is unrolled K times and they rotate at compile time.
 // The same by a whole warp: the K^2 rows' x passes on its lanes, the y pass of source plane c
 // on lane c, the z pass on every lane, with the same operations in the same order.  A short
 // list (a brick's last voxels) then takes one load latency instead of K^2.
@@ -194,6 +192,8 @@ __device__ __noinline__ unsigned dot2_voxel_warp(const void* src, int nx, int ny
     return comp_code(zs, zc, G.a0h, G.a0l, G.a1h, G.a1l, G.qmax);
 }
 
+// ROTZ: as in brick(); the accumulator slots are shifted after each plane, or the plane loop
+// is unrolled K times and they rotate at compile time.
 template <int K, int SF, class Wt, int LM = LM_ANY, bool ROI = false, bool ROTZ = true, bool BULK = false>
 __device__ __forceinline__ bool brick_split(const Job& J, const Wt& G, const CUtensorMap* tmap,
                                             int bx, int by, int bz, unsigned char* smem,

@@ -146,8 +146,9 @@ vktError launch_k(const Job& job, const float* gx, const float* gy, const float*
                                      Geo::raw_w(job.sfmt), ty + 2 * Geo::R, 1)
                     ? 1
                     : 0;
-    // rows that no tensor map can describe are still fetched asynchronously, as 16-byte
-    // blocks, when the volume starts on a 16-byte boundary
+    // rows that no tensor map can describe are still fetched asynchronously when the volume starts
+    // on a 16-byte boundary: as 16-byte blocks by the kernels of an integer format, else one bulk
+    // copy per row (copy_rows)
     J.rows = (!J.use_tma && reinterpret_cast<uintptr_t>(J.src) % 16 == 0) ? 1 : 0;
     if (!J.use_tma) memset(&map, 0, sizeof(map));
     size_t smem = J.comp ? sep::smem_bytes_comp<K>(job.sfmt, J.rows != 0)
