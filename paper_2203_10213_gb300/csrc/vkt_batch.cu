@@ -368,7 +368,7 @@ vktError build_plan(Plan& P, int32_t n, vktStructuredVolume* dst, vktStructuredV
         J.nz = s->dims[2];
         sep::set_whole_volume(J);
         J.sfmt = s->format;
-        J.dfmt = dst[i]->format;
+        J.dfmt = store_format(dst[i]->format, dst[i]->data);
         J.k = filters[i]->k;
         J.comp = modes[j] != B_PLAIN ? 1 : 0;   // (the split brick has the compensated one's tile)
         vnarrow[j] = narrow && modes[j] != B_SPLIT && narrow_for(J.nx, J.ny, J.comp != 0);

@@ -296,7 +296,6 @@ __device__ __forceinline__ void direct_body(const CUtensorMap& tmap, const Direc
     const int ox = x0 + tx * RX;
     const int nvalid = (ROI ? p.sx1 : p.nx) - ox;
     const int first = (ROI && p.sx0 > ox) ? p.sx0 - ox : 0;   // leading columns outside the region
-    const int nwide = wide_count(dst, nvalid);
     const int yend = ROI ? p.sy1 : p.ny;
     bool failed = false;
 
@@ -562,7 +561,7 @@ __device__ __forceinline__ void direct_body(const CUtensorMap& tmap, const Direc
                 for (int x = 0; x < RX; ++x) row[x] = lane(sl0, i, x);
                 if (oy < yend && nvalid > 0) {
                     const int64_t idx = (static_cast<int64_t>(oz) * p.ny + oy) * p.nx + ox;
-                    store_row<RX>(dst, dfmt, idx, nvalid, row, p.a0, p.a1, p.qmax, first, nwide);
+                    store_row<RX, (DF >= 0)>(dst, dfmt, idx, nvalid, row, p.a0, p.a1, p.qmax, first);
                 }
             }
         }
@@ -820,7 +819,7 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx, const ListPlan
     a.ny = job.ny;
     a.nz = job.nz;
     a.sfmt = job.sfmt;
-    a.dfmt = job.dfmt;
+    a.dfmt = store_format(job.dfmt, job.dst, job.nvol > 1 ? job.vs_dst : 0);
     a.a0 = job.a0;
     a.a1 = job.a1;
     a.qmax = job.qmax;
@@ -906,30 +905,30 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx, const ListPlan
     }
     if constexpr (!ADJ && MODE == M_PLAIN && K >= 3 && K <= 5) {
         // region tensor-map jobs of the common float32 destinations: formats compiled in
-        if (job.roi && a.use_tma && job.dfmt == FMT_F32 && job.sfmt == FMT_U8)
+        if (job.roi && a.use_tma && a.dfmt == FMT_F32 && job.sfmt == FMT_U8)
             kern = k_direct<K, ADJ, FMT_U8, FMT_F32, LM_TMA, true, M_PLAIN, SHAPE>;
-        if (job.roi && a.use_tma && job.dfmt == FMT_F32 && job.sfmt == FMT_F32)
+        if (job.roi && a.use_tma && a.dfmt == FMT_F32 && job.sfmt == FMT_F32)
             kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_TMA, true, M_PLAIN, SHAPE>;
     }
     if constexpr (ADJ && K >= 3 && K <= 5) {
         // the adjoint reads and writes float32: formats compiled in for tensor-map jobs
-        if (a.use_tma) kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_TMA, false, M_PLAIN, SHAPE>;
+        if (a.use_tma && a.dfmt == FMT_F32) kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_TMA, false, M_PLAIN, SHAPE>;
     }
     if constexpr (!ADJ && MODE == M_PLAIN && K >= 3 && K <= 5) {
-        if (!job.roi && job.dfmt == FMT_F32 && job.sfmt == FMT_U8) {
+        if (!job.roi && a.dfmt == FMT_F32 && job.sfmt == FMT_U8) {
             if (a.use_tma) kern = k_direct<K, ADJ, FMT_U8, FMT_F32, LM_TMA, false, M_PLAIN, SHAPE>;
             else if (a.rows) kern = k_direct<K, ADJ, FMT_U8, FMT_F32, LM_ROWS, false, M_PLAIN, SHAPE>;
         }
         // (not in the small shape: 59x200x210 16 us with run-time formats, 19 with these)
-        if (SHAPE == 0 && !job.roi && job.dfmt == FMT_U8 && job.sfmt == FMT_U8) {
+        if (SHAPE == 0 && !job.roi && a.dfmt == FMT_U8 && job.sfmt == FMT_U8) {
             if (a.use_tma) kern = k_direct<K, ADJ, FMT_U8, FMT_U8, LM_TMA, false, M_PLAIN, SHAPE>;
             else if (a.rows) kern = k_direct<K, ADJ, FMT_U8, FMT_U8, LM_ROWS, false, M_PLAIN, SHAPE>;
         }
-        if (SHAPE == 0 && !job.roi && job.dfmt == FMT_F32 && job.sfmt == FMT_U16) {
+        if (SHAPE == 0 && !job.roi && a.dfmt == FMT_F32 && job.sfmt == FMT_U16) {
             if (a.use_tma) kern = k_direct<K, ADJ, FMT_U16, FMT_F32, LM_TMA, false, M_PLAIN, SHAPE>;
             else if (a.rows) kern = k_direct<K, ADJ, FMT_U16, FMT_F32, LM_ROWS, false, M_PLAIN, SHAPE>;
         }
-        if (!job.roi && job.dfmt == FMT_F32 && job.sfmt == FMT_F32) {
+        if (!job.roi && a.dfmt == FMT_F32 && job.sfmt == FMT_F32) {
             if (a.use_tma) kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_TMA, false, M_PLAIN, SHAPE>;
             else if (a.rows) kern = k_direct<K, ADJ, FMT_F32, FMT_F32, LM_ROWS, false, M_PLAIN, SHAPE>;
         }

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(NT, 4)
         for (int it = 0; it < STAGES && it < nplanes; ++it) issue(it);
 
     const int gx = x0 + 4 * lane, gy = y0 + warp * RY;
-    const int nvalid = p.nx - gx, nwide = wide_count(dst, nvalid);
+    const int nvalid = p.nx - gx;
     const bool lface = x0 == 0, rface = x0 + TX - 1 + R > p.nx - 1;   // the tile touches a face
     // rows of the thread's windows, clamped to the volume, as stage offsets of their first voxel
     int off[RY + K - 1];
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(NT, 4)
                 if (oy < p.ny) {
                     const int64_t idx = (static_cast<int64_t>(pfirst + it - R) * p.ny + oy) * p.nx + gx;
                     const float v[4] = {acc[sl0][i][0].x, acc[sl0][i][0].y, acc[sl0][i][1].x, acc[sl0][i][1].y};
-                    store_row<4>(dst, FMT_F32, idx, nvalid, v, p.a0, p.a1, p.qmax, 0, nwide);
+                    store_row<4>(dst, FMT_F32, idx, nvalid, v, p.a0, p.a1, p.qmax);
                 }
             }
         }
@@ -173,14 +173,15 @@ __global__ void __launch_bounds__(NT, 4)
 }  // namespace
 
 // Launches the march where it serves the job: *taken false otherwise.  Whole float32 volumes (a batch
-// of them evenly spaced) that a tensor map describes, into float32, at least one tile (128 columns)
-// wide with three quarters of the tiles' columns in use, and large enough that 128 x 16 tiles in chunks
+// of them evenly spaced) that a tensor map describes, into float32 on 16 bytes, at least one tile (128
+// columns) wide with three quarters of the tiles' columns in use, and large enough that 128 x 16 tiles in chunks
 // of 8 planes give every SM its four CTAs; smaller ones have the one-row shape of the general kernel.
 vktError launch_march3(const Job& job, const float* w, const Ctx& ctx, bool* taken)
 {
     *taken = false;
-    if (job.roi || job.sfmt != FMT_F32 || job.dfmt != FMT_F32 || job.nx < TX) return VKT_NO_ERROR;
     const int nvol = std::max(job.nvol, 1);
+    if (job.roi || job.sfmt != FMT_F32 || job.nx < TX) return VKT_NO_ERROR;
+    if (store_format(job.dfmt, job.dst, nvol > 1 ? job.vs_dst : 0) != FMT_F32) return VKT_NO_ERROR;
     const int tx = (job.nx + TX - 1) / TX, ty = (job.ny + TY - 1) / TY;
     if (4 * static_cast<long>(job.nx) < 3L * tx * TX) return VKT_NO_ERROR;
     if (static_cast<long>(tx) * ty * (job.nz / 8) * nvol < 4L * ctx.sms) return VKT_NO_ERROR;

@@ -42,7 +42,7 @@ struct Job {
     const void* src;
     void* dst;
     int nx, ny, nz;
-    int sfmt, dfmt;
+    int sfmt, dfmt;    // dfmt: store_format
     int zchunk;
     int use_tma;
     int rows;          // no tensor map: stages filled by row copies (issue_rows)
@@ -249,7 +249,6 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
     const int ox = x0 + tx * RX;
     const int nvalid = (ROI ? J.sx1 : J.nx) - ox;
     const int first = (ROI && J.sx0 > ox) ? J.sx0 - ox : 0;   // leading columns outside the region
-    const int nwide = wide_count(J.dst, nvalid);
     const int yend = ROI ? J.sy1 : J.ny;
     bool failed = false;
 
@@ -414,7 +413,7 @@ __device__ __forceinline__ bool brick(const Job& J, const Wt& G, const CUtensorM
             const int oy = y0 + ty * RY + i;
             if (it >= 2 * R && oy < yend && nvalid > 0) {
                 const int64_t idx = (static_cast<int64_t>(pfirst + it - R) * J.ny + oy) * J.nx + ox;
-                store_row<RX, (K < 9)>(J.dst, dfmt, idx, nvalid, rowv, J.a0, J.a1, J.qmax, first, nwide);
+                store_row<RX, (K < 9 && !BULK)>(J.dst, dfmt, idx, nvalid, rowv, J.a0, J.a1, J.qmax, first);
             }
         };
         if constexpr (PAIR) {

@@ -110,7 +110,7 @@ vktError launch_k(const Job& job, const float* gx, const float* gy, const float*
     J.ny = job.ny;
     J.nz = job.nz;
     J.sfmt = job.sfmt;
-    J.dfmt = job.dfmt;
+    J.dfmt = store_format(job.dfmt, job.dst);
     J.k = K;
     J.a0 = job.a0;
     J.a1 = job.a1;

@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(NT, 2)
                         make_float4(fmaf(p.a1, v[0], p.a0), fmaf(p.a1, v[1], p.a0), fmaf(p.a1, v[2], p.a0),
                                     fmaf(p.a1, v[3], p.a0));
                 } else if constexpr (OUT == OUT_FP32_CODE) {
-                    store_row<4>(p.dst, p.dfmt, idx, 4, v, p.a0, p.a1, p.qmax, 0, 4);
+                    store_row<4>(p.dst, p.dfmt, idx, 4, v, p.a0, p.a1, p.qmax);
                 } else {
                     unsigned code[4];
 #pragma unroll

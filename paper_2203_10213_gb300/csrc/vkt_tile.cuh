@@ -11,6 +11,19 @@ namespace vkt {
 
 enum : int { FMT_U8 = 0, FMT_U16 = 1, FMT_F32 = 2 };
 
+// A kernel's float32 destination that does not start on 16 bytes: stored voxel by voxel.  With
+// FMT_F32 the launcher vouches for the alignment, so a row is stored as one by its index alone (a count
+// kept for it in every thread cost 256x256x128 float32 dense k = 3 21.5 -> 22.4 us, a batch of 96 float32
+// volumes at k = 7 344 -> 372).
+constexpr int FMT_F32_SCALAR = 3;
+
+// The destination format of a launch; vs: voxels from one volume's destination to the next.
+inline int store_format(int dfmt, const void* dst, int64_t vs = 0)
+{
+    const bool wide = ((reinterpret_cast<uintptr_t>(dst) | static_cast<uintptr_t>(4 * vs)) & 15) == 0;
+    return dfmt == FMT_F32 && !wide ? FMT_F32_SCALAR : dfmt;
+}
+
 constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;   // 2 s for any single device wait
 
 __host__ __device__ constexpr int fmt_bytes(int f) { return f == FMT_U8 ? 1 : (f == FMT_U16 ? 2 : 4); }
@@ -508,31 +521,27 @@ __device__ __forceinline__ void store_codes(void* dst, int dfmt, int64_t idx, in
     }
 }
 
-// How many results of a row may be stored as one: those of a float32 destination that starts on a
-// 16-byte boundary (store_row then needs to look at the row's own offset only).
-__device__ __forceinline__ int wide_count(const void* dst, int nvalid)
-{
-    return (reinterpret_cast<uintptr_t>(dst) & 15) == 0 ? nvalid : 0;
-}
-
 // Writes results first .. nvalid-1 of RX consecutive results of one row (from idx), mapped
-// to the destination format; nwide: wide_count(dst, nvalid).
-// WIDE: codes are stored as a word where they are aligned.  Not in the separable brick at k = 9, whose
-// plane loop is unrolled nine times: the added code costs its instruction fetch more than the stores
-// save (45x458x151 uint8, a region of interest, 41.3 against 39.6 us, into float32 39.8 against 38.3).
+// to the destination format (store_format).
+// WIDE: codes are stored as a word where they are aligned.  Not where the added code costs more
+// instruction fetch than the stores save: in the separable brick at k = 9, whose plane loop is
+// unrolled nine times (45x458x151 uint8, a region of interest, 41.3 against 39.6 us, into float32 39.8
+// against 38.3), in the batch's bricks (96 uint8 volumes of 16 to 256 per axis, k = 5 347 against 322
+// us, k = 7 387 against 357) and in the direct kernels with the format chosen at run time (203x190x180
+// uint8, k = 1 25.6 against 22.9).
 template <int RX, bool WIDE = true>
 __device__ __forceinline__ void store_row(void* dst, int dfmt, int64_t idx, int nvalid,
                                           const float (&acc)[RX], float a0, float a1, float qmax,
-                                          int first, int nwide)
+                                          int first = 0)
 {
     float v[RX];
 #pragma unroll
     for (int x = 0; x < RX; ++x) v[x] = fmaf(a1, acc[x], a0);
-    if (dfmt == FMT_F32) {
+    if (dfmt >= FMT_F32) {
         float* d = reinterpret_cast<float*>(dst) + idx;
-        if (RX == 4 && first == 0 && nwide >= 4 && (idx & 3) == 0) {
+        if (RX == 4 && dfmt == FMT_F32 && first == 0 && nvalid >= 4 && (idx & 3) == 0) {
             *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
-        } else if (RX == 2 && first == 0 && nwide >= 2 && (idx & 1) == 0) {
+        } else if (RX == 2 && dfmt == FMT_F32 && first == 0 && nvalid >= 2 && (idx & 1) == 0) {
             *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
         } else {
 #pragma unroll

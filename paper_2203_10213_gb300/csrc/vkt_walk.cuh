@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(NT, 3)
         for (int it = 0; it < STAGES && it < nplanes; ++it) issue(it);
 
     const int gx = x0 + 4 * lane, gy = y0 + warp * RY;
-    const int nvalid = p.nx - gx, nwide = wide_count(p.dst, nvalid);
+    const int nvalid = p.nx - gx;
     const bool lface = x0 == 0, rface = x0 + TX - 1 + R > p.nx - 1;   // the tile touches a face
     // rows of the thread's windows, clamped to the volume, as stage offsets of their first columns
     int off[RY + K - 1];
@@ -208,8 +208,7 @@ __global__ void __launch_bounds__(NT, 3)
                 if (oy < p.ny) {
                     const int64_t idx = (static_cast<int64_t>(pfirst + it - R) * p.ny + oy) * p.nx + gx;
                     const float v[4] = {acc[sl0][i][0].x, acc[sl0][i][0].y, acc[sl0][i][1].x, acc[sl0][i][1].y};
-                    store_row<4>(p.dst, OUT_F32 ? FMT_F32 : p.dfmt, idx, nvalid, v, p.a0, p.a1, p.qmax, 0,
-                                 nwide);
+                    store_row<4>(p.dst, OUT_F32 ? FMT_F32 : p.dfmt, idx, nvalid, v, p.a0, p.a1, p.qmax);
                 }
             }
         }
@@ -268,9 +267,7 @@ vktError launch_walk_k(const Job& job, const float* gx, const float* gy, const f
     size_t smem = 0;
     auto pick = [&](auto sf) {
         constexpr int SF = decltype(sf)::value;
-        kern = k_walk<K, SF, true>;
-        if constexpr (SF != FMT_F32)
-            if (job.dfmt != FMT_F32) kern = k_walk<K, SF, false>;
+        kern = store_format(job.dfmt, job.dst) == FMT_F32 ? k_walk<K, SF, true> : k_walk<K, SF, false>;
         smem = Cfg<K, SF>::SMEM;
     };
     if (job.sfmt == FMT_F32) pick(std::integral_constant<int, FMT_F32>{});
@@ -286,7 +283,7 @@ vktError launch_walk_k(const Job& job, const float* gx, const float* gy, const f
     a.nx = job.nx;
     a.ny = job.ny;
     a.nz = job.nz;
-    a.dfmt = job.dfmt;
+    a.dfmt = store_format(job.dfmt, job.dst);
     a.a0 = job.a0;
     a.a1 = job.a1;
     a.qmax = job.qmax;
