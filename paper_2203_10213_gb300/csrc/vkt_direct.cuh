@@ -66,6 +66,7 @@ constexpr int LIST_AT = 512;     // listed voxels that are worked off once there
 constexpr int NT = 256;          // threads per CTA, 16 x 16
 constexpr int BX = 16, BY = 16;
 constexpr int STAGES = 4;        // raw tiles in flight per CTA
+constexpr size_t SM_SMEM = 228 * 1024, SM_SMEM_PER_CTA = 1024;   // of an SM; what a CTA takes besides its own
 
 template <int K>
 struct DenseW {
@@ -893,7 +894,7 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx, const ListPlan
                  ? 1
                  : 0;
 
-    const size_t smem = direct_smem_bytes<K, MODE, SHAPE>(job.sfmt, a.rows != 0);
+    size_t smem = direct_smem_bytes<K, MODE, SHAPE>(job.sfmt, a.rows != 0);
     // the common pairs of formats get kernels with them compiled in (k = 3, 302^3 uint8
     // into uint8 95 -> 79, 256x256x200 30 -> 28 us); tensor-map jobs get kernels without the
     // other ways of loading, and so do row-copy jobs of the compiled-in formats; plain-load
@@ -941,11 +942,28 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx, const ListPlan
                               : zchunk_direct(static_cast<long>(gx) * gy * nvol, a.ez, sms, per_sm, R);
     const int gz = (a.ez + a.zchunk - 1) / a.zchunk;
     a.gzv = gz;
+    // A launch of less than a wave: as much shared memory as lets no more CTAs onto an SM than an even
+    // spread needs.  CTAs of the next call come in while those of the one before still hold their places
+    // (programmatic launch), so without it some SMs take all they have room for and the others few; the
+    // fewer registers a kernel takes, the worse.  us, kernel before it took fewer registers / without /
+    // with this: uint16 k = 5 100x64x300 30 / 37 / 27, 45x458x151 48 / 60 / 44; region 192x192x96 float32
+    // k = 3 13.6 / 15.7 / 12.0, uint16 codes k = 1 15.3 / 18.1 / 13.0.  Not Dot2 at k = 3, whose warps are
+    // few already (100x64x300 float32 into codes 41.3, with this 43.4).
+    const long even = (static_cast<long>(gx) * gy * gz * nvol + sms - 1) / sms;
+    if (even < per_sm && !(MODE == M_DOT2 && K == 3)) {
+        const size_t share = (SM_SMEM / (even + 1) - SM_SMEM_PER_CTA + 128) & ~static_cast<size_t>(127);
+        int fit = 0;
+        if (share > smem && prepare_kernel(ctx, reinterpret_cast<const void*>(kern), NT, share, &fit) == VKT_NO_ERROR &&
+            fit == even) {
+            smem = share;
+            per_sm = fit;
+        }
+    }
     const int per_launch = std::max(1, 65535 / gz);
     if (a.use_tma && per_launch < nvol && !encode(job.src, per_launch)) return VKT_ERROR_CUDA;
     if (ctx.debug & VKT_DEBUG_LOG)
-        fprintf(stderr, "[vkt] direct%s k=%d grid=(%d,%d,%d) zchunk=%d smem=%zu tma=%d rows=%d withhold=%d\n",
-                ADJ ? "-adjoint" : (MODE == M_DOT2 ? "-compensated" : MODE == M_LIST ? "-listed" : MODE == M_PAIR ? "-listed-pair" : ""), K, gx, gy, gz, a.zchunk, smem,
+        fprintf(stderr, "[vkt] direct%s k=%d grid=(%d,%d,%d) zchunk=%d smem=%zu per_sm=%d tma=%d rows=%d withhold=%d\n",
+                ADJ ? "-adjoint" : (MODE == M_DOT2 ? "-compensated" : MODE == M_LIST ? "-listed" : MODE == M_PAIR ? "-listed-pair" : ""), K, gx, gy, gz, a.zchunk, smem, per_sm,
                 a.use_tma, a.rows, a.withhold_first);
     const DirectArgs a0 = a;
     for (int v0 = 0; v0 < nvol; v0 += per_launch) {

@@ -792,11 +792,10 @@ static std::string tune_key(const vktStructuredVolume_impl* dst, const vktStruct
 // CTA per SM) 1.03 us, and 8.5 us for the launch, the first plane and the last; on the direct path
 // (64 x 32 columns) 1.86, 3.03 or 4.05 us with one, two or three CTAs on that SM.  Measured over 174
 // cases of 1 to 8 volumes of 32^3 to 1024x1024x256, powers of two and not, these are within 10 % of
-// the times, and the path chosen is never the slower one by more than 2 %.  us, direct / tensor:
-// 64^3 9.3 / 20.6, four of them
-// 24.8 / 20.7; eight of 160x32x128 48.8 / 92.7 (a quarter of each tensor tile in use), of 132x100x96
-// 112 / 60, of 128^3 93 / 81; one 160x150x128 48 / 33 and eight 182 / 192; 512^3 620 / 499.
-// (At k = 7 the tensor path is the faster one throughout: two of 32^3 30.7 / 24.8.)
+// the times, and the path chosen is never the slower one by more than 3.5 %.  us, direct / tensor:
+// 64^3 9.3 / 20.6, eight of them 23.9 / 28.8; 128^3 24.0 / 20.7, eight 93 / 81; eight of 160x32x128
+// 49 / 93 (a quarter of each tensor tile in use), of 132x100x96 112 / 59, of 160x150x128 181 / 192;
+// 512^3 619 / 499.  (At k = 7 the tensor path is the faster one throughout: two of 32^3 31 / 25.)
 static bool direct5_faster(const int32_t* dims, long n)
 {
     int dev = 0, sms = 152;
@@ -810,7 +809,7 @@ static bool direct5_faster(const int32_t* dims, long n)
     const long tiles = over(nx, 64) * over(ny, 32) * n;
     const long dz = zchunk_direct(tiles, nz, sms, 3, 2);
     const long ctas = tiles * over(nz, dz);
-    const double plane = ctas <= sms ? 1.86 : 2 * ctas <= 3L * sms ? 3.03 : 4.05;
+    const double plane = ctas <= sms ? 1.86 : ctas <= 2L * sms ? 3.03 : 4.05;
     return plane * static_cast<double>(over(ctas, 3L * sms) * (dz + 4)) < tensor;
 }
 

@@ -49,7 +49,7 @@ def paths(capfd, call):
 
 # n, (nz, ny, nx), launches on the tensor and on the direct path
 @pytest.mark.parametrize("n,shape,want", [(1, (64, 64, 64), (0, 1)), (2, (32, 32, 32), (0, 1)),
-                                          (4, (64, 64, 64), (1, 0)), (1, (128, 128, 128), (1, 0)),
+                                          (4, (64, 64, 64), (0, 1)), (1, (128, 128, 128), (1, 0)),
                                           (8, (128, 128, 128), (1, 0)), (4, (96, 100, 132), (1, 0)),
                                           (8, (128, 32, 160), (0, 1)), (1, (96, 100, 132), (1, 0))])
 def test_path_by_rule(n, shape, want, capfd):
