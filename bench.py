@@ -78,8 +78,9 @@ KERNEL_CASES = {
 # used only while the sources are unchanged.
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.md")
 KERNEL_SOURCES = {
-    "separable gaussian5": ["vkt_sep_brick.cuh", "vkt_separable.cuh", "vkt_separable5.cu", "vkt_tile.cuh"],
-    "direct laplacian3": ["vkt_direct.cuh", "vkt_direct.cu", "vkt_tile.cuh"],
+    "separable gaussian5": ["vkt_sep_brick.cuh", "vkt_separable.cuh", "vkt_separable5.cu", "vkt_tile.cuh",
+                            "vkt_window.cuh"],
+    "direct laplacian3": ["vkt_star.cu", "vkt_tile.cuh", "vkt_window.cuh"],
 }
 
 
