@@ -920,12 +920,13 @@ vktError launch_k(const Job& job, const float* w, const Ctx& ctx, const ListPlan
             if (a.use_tma) kern = k_direct<K, ADJ, FMT_U8, FMT_F32, LM_TMA, false, M_PLAIN, SHAPE>;
             else if (a.rows) kern = k_direct<K, ADJ, FMT_U8, FMT_F32, LM_ROWS, false, M_PLAIN, SHAPE>;
         }
-        // (not in the small shape: 59x200x210 16 us with run-time formats, 19 with these)
-        if (SHAPE == 0 && !job.roi && a.dfmt == FMT_U8 && job.sfmt == FMT_U8) {
+        // (in the small shape too: uint8 into uint8 96^3 5.9 us with run-time formats, 5.4 with these,
+        // 45x100x60 6.4 and 5.4; uint16 into float32 5.7 and 5.1, 6.3 and 5.4)
+        if (!job.roi && a.dfmt == FMT_U8 && job.sfmt == FMT_U8) {
             if (a.use_tma) kern = k_direct<K, ADJ, FMT_U8, FMT_U8, LM_TMA, false, M_PLAIN, SHAPE>;
             else if (a.rows) kern = k_direct<K, ADJ, FMT_U8, FMT_U8, LM_ROWS, false, M_PLAIN, SHAPE>;
         }
-        if (SHAPE == 0 && !job.roi && a.dfmt == FMT_F32 && job.sfmt == FMT_U16) {
+        if (!job.roi && a.dfmt == FMT_F32 && job.sfmt == FMT_U16) {
             if (a.use_tma) kern = k_direct<K, ADJ, FMT_U16, FMT_F32, LM_TMA, false, M_PLAIN, SHAPE>;
             else if (a.rows) kern = k_direct<K, ADJ, FMT_U16, FMT_F32, LM_ROWS, false, M_PLAIN, SHAPE>;
         }
